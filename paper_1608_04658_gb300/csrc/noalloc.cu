@@ -13,7 +13,7 @@
 // as it does every other device pointer the caller holds).
 #include <mutex>
 
-#include "lbm_internal.cuh"
+#include "totals.cuh"
 
 namespace lbm {
 
@@ -32,26 +32,19 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) noalloc_partial_kernel(const 
 {
     const long long beg = (long long)blockIdx.x * NOALLOC_CHUNK;
     const long long end = beg + NOALLOC_CHUNK < N ? beg + NOALLOC_CHUNK : N;
-    double acc[5] = {0, 0, 0, 0, 0};
+    using R = typename Codec<S>::R;
+    NodeTotals<R> T;
     for (long long n = beg + threadIdx.x; n < end; n += NOALLOC_THREADS) {
         if (flags && (flags[n] & FL_SOLID)) continue;
-        double r = 0, j[3] = {0, 0, 0};
-        for (int i = 0; i < Q; ++i) {
-            const double v = (double)Codec<S>::load(f + (size_t)i * N + n) + weight<double>(i) * rho0;
-            r += v;
-            j[0] += cx_of(i) * v;
-            j[1] += cy_of(i) * v;
-            j[2] += cz_of(i) * v;
-        }
-        acc[0] += r;
-        acc[1] += j[0];
-        acc[2] += j[1];
-        acc[3] += j[2];
-        acc[4] += 0.5 * (j[0] * j[0] + j[1] * j[1] + j[2] * j[2]) / r;
+        R g[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) g[i] = Codec<S>::load(f + (size_t)i * N + n);
+        T.add(g, rho0);
     }
+    T.finish(rho0);
     __shared__ double sm[NOALLOC_THREADS / 32][5];
     for (int k = 0; k < 5; ++k) {
-        double v = acc[k];
+        double v = T.acc[k];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5][k] = v;
     }

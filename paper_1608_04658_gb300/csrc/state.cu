@@ -5,6 +5,7 @@
 #include <type_traits>
 
 #include "kbc.cuh"
+#include "totals.cuh"
 
 namespace lbm {
 
@@ -59,27 +60,20 @@ __global__ void __launch_bounds__(256) totals_kernel(const Lattice L, const S *_
                                                      const uint8_t *__restrict__ flags,
                                                      double *__restrict__ partials)
 {
-    double acc[5] = {0, 0, 0, 0, 0};
+    using R = typename Codec<S>::R;
+    NodeTotals<R> T;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < L.N;
          n += (long long)gridDim.x * blockDim.x) {
         if (flags && (flags[n] & FL_SOLID)) continue;
-        double r = 0, j[3] = {0, 0, 0};
-        for (int i = 0; i < Q; ++i) {
-            const double v = (double)Codec<S>::load(f + (size_t)i * L.N + n) + weight<double>(i) * L.rho0;
-            r += v;
-            j[0] += cx_of(i) * v;
-            j[1] += cy_of(i) * v;
-            j[2] += cz_of(i) * v;
-        }
-        acc[0] += r;
-        acc[1] += j[0];
-        acc[2] += j[1];
-        acc[3] += j[2];
-        acc[4] += 0.5 * (j[0] * j[0] + j[1] * j[1] + j[2] * j[2]) / r;
+        R g[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) g[i] = Codec<S>::load(f + (size_t)i * L.N + n);
+        T.add(g, L.rho0);
     }
+    T.finish(L.rho0);
     __shared__ double sm[8][5];
     for (int k = 0; k < 5; ++k) {
-        double v = acc[k];
+        double v = T.acc[k];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5][k] = v;
     }
