@@ -303,7 +303,7 @@ class Lattice:
             raise LbmError(st, "lbm_create failed")
         self._ctx = ctx
         self._keep = []
-        self._dependents = []  # weak references to the refinements that use this lattice
+        self._dependents = []  # references to the refinements that use this lattice (called for the object to close)
 
     # -------------------------------------------------------------- helpers
     def _check(self, st: int):
@@ -608,6 +608,24 @@ def fine_nu(nu: float) -> float:
     return 2.0 * float(nu)
 
 
+class _RefineHandle:
+    """The library's refinement, shared by the Refinement and its two levels:
+    whichever of the three is finalised first destroys it, whatever the order
+    (the garbage collector finalises the objects of a cycle in any order, and
+    clears weak references between them beforehand)."""
+
+    def __init__(self, ptr):
+        self.ptr = ptr
+
+    def __call__(self):
+        return self
+
+    def close(self):
+        ptr, self.ptr = self.ptr, None
+        if ptr:
+            lib().lbm_refine_destroy(ptr)
+
+
 class Refinement:
     """Two-level block refinement (lbm_refine_*; Sec. 4.2's two-level grid).
 
@@ -636,14 +654,20 @@ class Refinement:
             self.fine.close()  # nothing refers to it yet: give its memory back now
             raise err
         self._r = r
-        import weakref
-        coarse._dependents.append(weakref.ref(self))
-        self.fine._dependents.append(weakref.ref(self))
+        coarse._dependents.append(self._handle)
+        self.fine._dependents.append(self._handle)
+
+    @property
+    def _r(self):
+        return self._handle.ptr
+
+    @_r.setter
+    def _r(self, ptr):
+        self._handle = _RefineHandle(ptr)
 
     def close(self):
-        if getattr(self, "_r", None):
-            lib().lbm_refine_destroy(self._r)
-            self._r = None
+        if getattr(self, "_handle", None):
+            self._handle.close()
 
     def __del__(self):
         try:

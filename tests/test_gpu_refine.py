@@ -330,3 +330,26 @@ def test_refined_run_resumes_bitwise(tmp_path):
     with pytest.raises(lbm.LbmError) as e:
         ref3.load(pr)
     assert e.value.status == binding.LBM_ERR_ARG
+
+
+def test_refinement_in_a_garbage_cycle():
+    """The collector may finalise the levels of an unreachable refinement
+    before the refinement itself: the library's coupling goes first all the same."""
+    import gc
+
+    import paper_1608_04658_gb300 as lbm
+    destroyed = []
+    L = lbm.lib()
+    for first in ("lat", "ref"):
+        lat = lbm.Lattice((24, 20, 18), 0.02, storage="fp32")
+        ref = lbm.Refinement(lat, (5, 4, 3), (16, 13, 12))
+        handle = ref._handle
+        lat.cycle = ref  # reachable from each other only
+        if first == "lat":
+            lat.__del__()  # the order in which a weak reference to ref would already be dead
+            assert handle.ptr is None
+        del lat, ref
+        gc.collect()
+        assert handle.ptr is None
+        destroyed.append(first)
+    assert destroyed == ["lat", "ref"] and L is lbm.lib()
