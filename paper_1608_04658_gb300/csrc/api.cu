@@ -343,7 +343,16 @@ lbm_status lbm_set_geometry(lbm_ctx *ctx, const lbm_geometry *g)
         G.inv_chord = 1.0 / g->chord;
         G.camber_k1 = g->camber_p > 0.0 ? g->camber_m / (g->camber_p * g->camber_p) : 0.0;
         G.camber_k2 = g->camber_p < 1.0 ? g->camber_m / ((1.0 - g->camber_p) * (1.0 - g->camber_p)) : 0.0;
-        for (int k = 0; k < 5; ++k) G.thick[k] = g->thick[k];
+        for (int k = 0; k < 5; ++k) {
+            G.thick[k] = g->thick[k];
+            G.thick_f[k] = (float)g->thick[k];
+        }
+        G.camber_p_f = (float)G.camber_p;
+        G.camber_k1_f = (float)G.camber_k1;
+        G.camber_k2_f = (float)G.camber_k2;
+        double mag = 1.0 + std::fabs(G.camber_k1) + std::fabs(G.camber_k2);
+        for (double t : G.thick) mag += std::fabs(t);
+        G.sure_f = (float)(1e-4 * mag);
         G.y_base = g->X[1];
         // profile box in the lattice frame (relative to the leading edge) from a
         // dense sample of the outline, widened by one node
@@ -462,7 +471,7 @@ lbm_status lbm_set_geometry(lbm_ctx *ctx, const lbm_geometry *g)
     G.cap_boundary = (int)vol;
     G.cap_uncovered = (int)vol;
     Scratch &S = ctx->S;
-    S.n_partials = 64;
+    S.n_partials = FORCE_BLOCKS;
     bool ok = true;
     if (body) {
         ok = ctx_alloc(ctx, &S.blist, vol) == cudaSuccess && ctx_alloc(ctx, &S.bpos, vol) == cudaSuccess &&
@@ -586,7 +595,7 @@ static cudaError_t sequential_step(lbm_ctx *ctx, void *fa, void *fb, int &cur, i
             (e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0)) != cudaSuccess ||
             (e = launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, ctx->flags, ctx->side)) !=
                 cudaSuccess ||
-            (e = launch_forces(ctx->G, ctx->S, cur, ctx->side, &launches)) != cudaSuccess ||
+            (e = launch_forces(ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches)) != cudaSuccess ||
             (e = cudaEventRecord(ctx->ev_join, ctx->side)) != cudaSuccess)
             return e;
         launches += 1;
@@ -683,7 +692,7 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
             LBM_CUDA(launch_geometry(ctx->L, ctx->G, ctx->S, prev, ctx->flags, ctx->side, &launches), "geometry");
             LBM_CUDA(launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, ctx->flags, ctx->side), "refill");
             LBM_CUDA(launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, ctx->flags, ctx->side), "boundary");
-            LBM_CUDA(launch_forces(ctx->G, ctx->S, cur, ctx->side, &launches), "forces");
+            LBM_CUDA(launch_forces(ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches), "forces");
             LBM_CUDA(launch_bulk(ctx->storage, ctx->L, fa, fb, ctx->flags, status, ctx->side, BULK_BAND, sweep,
                                  ctx->G.cap), "bulk band");
             LBM_CUDA(cudaEventRecord(ctx->ev_join, ctx->side), "join");
@@ -771,7 +780,7 @@ lbm_status lbm_step_edges(lbm_ctx *ctx)
         LBM_CUDA(launch_geometry(ctx->L, ctx->G, ctx->S, prev, ctx->flags, ctx->side, &launches), "geometry");
         LBM_CUDA(launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, ctx->flags, ctx->side), "refill");
         LBM_CUDA(launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, ctx->flags, ctx->side), "boundary");
-        LBM_CUDA(launch_forces(ctx->G, ctx->S, cur, ctx->side, &launches), "forces");
+        LBM_CUDA(launch_forces(ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches), "forces");
         LBM_CUDA(launch_bulk(ctx->storage, ctx->L, fa, fb, ctx->flags, status, ctx->side, BULK_BAND, sweep,
                              ctx->G.cap), "bulk band");
         LBM_CUDA(cudaEventRecord(ctx->ev_join, ctx->side), "join");

@@ -25,6 +25,10 @@ struct GeomParams {
     // airfoil
     double chord, ca, sa, h_amp, h_omega, camber_m, camber_p, thick[5], y_base;
     double inv_chord, camber_k1, camber_k2;  // 1/c, m/p^2, m/(1-p)^2 (single-precision link search)
+    // the profile rounded once to FP32: a conversion of each coefficient in
+    // every halving of a link runs at the FP64 rate
+    float thick_f[5], camber_p_f, camber_k1_f, camber_k2_f;
+    float sure_f;  // bound on the FP32 profile's error (chords, with a wide margin)
     double box[4];       // profile box relative to the leading edge: dx min/max, dy min/max
     // swimmer mesh (device arrays owned by Scratch)
     const double *mesh_rest;  // (s, dy, dz) per vertex
@@ -81,6 +85,8 @@ struct DevBody {
     int sweep[6];
 };
 
+constexpr int FORCE_BLOCKS = 128;   // blocks (and partial sums) of the force reduction
+
 // scratch owned by the library for the boundary path
 struct Scratch {
     DevBody *body;       // [2]
@@ -109,7 +115,8 @@ cudaError_t launch_refill(int storage, const Lattice &L, const GeomParams &G, Sc
                           void *fa, const uint8_t *flags, cudaStream_t s);
 cudaError_t launch_boundary(int storage, const Lattice &L, const GeomParams &G, Scratch &S, int cur,
                             const void *fa, void *fb, const uint8_t *flags, cudaStream_t s);
-cudaError_t launch_forces(const GeomParams &G, Scratch &S, int cur, cudaStream_t s, int *nlaunch);
+cudaError_t launch_forces(const Lattice &L, const GeomParams &G, Scratch &S, int cur, const uint8_t *flags,
+                          cudaStream_t s, int *nlaunch);
 cudaError_t launch_sweep_init(const Lattice &L, const GeomParams &G, Scratch &S, int cur, cudaStream_t s);
 struct Force6 {
     double v[6];

@@ -118,9 +118,10 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
             }
         }
         const R nmiss = R(__popc(mask));
-        const R rho_t = rho0 + wsum(act ? gstat : R(0)) + wsum(dyn);
-        R u_t[3];
-        for (int a = 0; a < 3; ++a) u_t[a] = wsum(ut[a]) / nmiss;
+        R t[6] = {act ? gstat : R(0), dyn, ut[0], ut[1], ut[2], R(0)};
+        wsum6(t, lane);
+        const R rho_t = rho0 + t[0] + t[1];
+        const R u_t[3] = {t[2] / nmiss, t[3] / nmiss, t[4] / nmiss};
         R du[3][3];
         const R uc[3] = {su[13][1], su[13][2], su[13][3]};
         fd_gradient<R>(su, sok, uc, du);
@@ -130,13 +131,16 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
         if (miss) gi = grad_shifted<R>(i, rho_t, rho0, u_t, Qt);
 
         // momentum exchange on missing links (FP64): the fluid hands the body
-        // (c_opp - u_w) f'_opp(x_b, t) and gets back (c_i - u_w) F_i(x_b, t+1)
+        // (c_opp - u_w) f'_opp(x_b, t) and gets back (c_i - u_w) F_i(x_b, t+1):
+        // -c_i (f_out + f_in) + u_w (f_in - f_out), in which W rho0 leaves the
+        // difference and c_i is a sign
         double dF[6] = {0, 0, 0, 0, 0, 0};
         if (miss) {
-            const double W = weight<double>(i) * L.rho0;
-            const double fout = (double)fbb + W, fin = (double)gi + W;
+            const double fo = (double)fbb, fi = (double)gi;
+            const double sum = (fo + fi) + 2.0 * weight<double>(i) * L.rho0, dif = fi - fo;
+            const int ci[3] = {cx, cy, cz};
+            for (int a = 0; a < 3; ++a) dF[a] = fma(uw[a], dif, ci[a] == 0 ? 0.0 : (ci[a] > 0 ? -sum : sum));
             const double c[3] = {(double)cx, (double)cy, (double)cz};
-            for (int a = 0; a < 3; ++a) dF[a] = (-c[a] - uw[a]) * fout - (c[a] - uw[a]) * fin;
             double r[3];
             r[0] = body_offset(L, G, b, 0, x) - q * c[0];
             r[1] = body_offset(L, G, b, 1, y) - q * c[1];
@@ -145,14 +149,13 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
             dF[4] = r[2] * dF[0] - r[0] * dF[2];
             dF[5] = r[0] * dF[1] - r[1] * dF[0];
         }
-        const int pos = bpos[slot];
         // a slab's links count where it owns the fluid node
         const bool own = z >= G.own_lo && z < G.own_hi;
-        for (int k = 0; k < 6; ++k) {
-            double v = dF[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-            if (lane == 0) bforce[(size_t)pos * 6 + k] = own ? v : 0.0;
-        }
+        const double fsum = wsum_scatter6(dF, lane);
+        const size_t pos = (size_t)bpos[slot] * 6;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (lane == wsum_owner6(k)) bforce[pos + k] = own ? fsum : 0.0;
 
         bool ok;
         const R out = kbc_collide_lanes<R>(gi, i, (R)L.beta, (R)L.inv_beta, rho0, L.gamma_mode, ok);

@@ -81,10 +81,32 @@ __device__ __forceinline__ bool inside_airfoil(const GeomParams &G, const double
     return fabs(__dsub_rn(eta, airfoil_camber(G, xi))) < airfoil_half_thickness(G, xi);
 }
 
+// The same decision, in FP32 wherever FP32 is far enough from the surface to be
+// sure of it: the double form's divisions and square root cost some 60 FP64
+// operations a node (two lanes a clock and SM), and only the nodes within some
+// 1e-4 chords of the outline need them.  The FP32 coordinates carry an error of
+// a few 1e-7 chords, the margin a few 1e-6 of the profile's coefficients (away
+// from the blunt nose, where the square root is steep: xi < 1e-3 is left to the
+// double form), against bounds of 1e-4 of them.
+__device__ __forceinline__ float airfoil_margin_f(const GeomParams &G, float xi, float eta);
+__device__ __forceinline__ bool inside_airfoil_fast(const GeomParams &G, const double X[3], double x, double y)
+{
+    const float dx = (float)__dsub_rn(x, X[0]), dy = (float)__dsub_rn(y, X[1]);
+    const float ca = (float)G.ca, sa = (float)G.sa, ic = (float)G.inv_chord;
+    const float xi = (dx * ca - dy * sa) * ic, eta = (dx * sa + dy * ca) * ic;
+    if (xi < -1e-4f || xi > 1.0f + 1e-4f) return false;
+    if (xi > 1e-3f && xi < 1.0f - 1e-4f) {
+        const float m = airfoil_margin_f(G, xi, eta);
+        if (m > G.sure_f) return true;
+        if (m < -G.sure_f) return false;
+    }
+    return inside_airfoil(G, X, x, y);
+}
+
 __device__ __forceinline__ bool inside_body(const GeomParams &G, const Lattice &L, const double X[3],
                                             int x, int y, int z)
 {
-    if (G.kind == LBM_BODY_AIRFOIL) return inside_airfoil(G, X, (double)x, (double)y);
+    if (G.kind == LBM_BODY_AIRFOIL) return inside_airfoil_fast(G, X, (double)x, (double)y);
     if (G.kind == LBM_BODY_SPHERE) {
         const double dx = axis_offset(x, X[0], L.nx, G.periodic[0]);
         const double dy = axis_offset(y, X[1], L.ny, G.periodic[1]);
@@ -343,15 +365,21 @@ __device__ void mesh_links_warp(const GeomParams &G, const DevBody *b, int x, in
 
 // airfoil link in the chord frame: node position and link direction in
 // double, the 24 halvings in float with reciprocal constants
+// (airfoil_margin_f: half thickness less the distance from the camber line)
+__device__ __forceinline__ float airfoil_margin_f(const GeomParams &G, float xi, float eta)
+{
+    const float p = G.camber_p_f;
+    const float yc = xi < p ? G.camber_k1_f * (2.0f * p * xi - xi * xi)
+                            : G.camber_k2_f * ((1.0f - 2.0f * p) + 2.0f * p * xi - xi * xi);
+    const float t = G.thick_f[0] * sqrtf(xi) +
+                    xi * (G.thick_f[1] + xi * (G.thick_f[2] + xi * (G.thick_f[3] + xi * G.thick_f[4])));
+    return t - fabsf(eta - yc);
+}
+
 __device__ __forceinline__ bool inside_airfoil_f(const GeomParams &G, float xi, float eta)
 {
     if (xi < 0.0f || xi > 1.0f) return false;
-    const float p = (float)G.camber_p;
-    const float yc = xi < p ? (float)G.camber_k1 * (2.0f * p * xi - xi * xi)
-                            : (float)G.camber_k2 * ((1.0f - 2.0f * p) + 2.0f * p * xi - xi * xi);
-    const float t = (float)G.thick[0] * sqrtf(xi) +
-                    xi * ((float)G.thick[1] + xi * ((float)G.thick[2] + xi * ((float)G.thick[3] + xi * (float)G.thick[4])));
-    return fabsf(eta - yc) < t;
+    return airfoil_margin_f(G, xi, eta) > 0.0f;
 }
 
 __device__ __forceinline__ double link_airfoil_f(const GeomParams &G, const DevBody *b, int x, int y, int cx, int cy)

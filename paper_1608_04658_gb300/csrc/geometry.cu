@@ -204,8 +204,7 @@ __device__ __forceinline__ bool band_node(const Lattice &L, const GeomParams &G,
 __global__ void __launch_bounds__(GEOM_THREADS) mark_kernel(const Lattice L, const GeomParams G,
                                                             const DevBody *__restrict__ prev,
                                                             DevBody *__restrict__ cur,
-                                                            uint8_t *__restrict__ flags,
-                                                            double *__restrict__ bforce)
+                                                            uint8_t *__restrict__ flags)
 {
     __shared__ double sX[3];
     __shared__ int slo[3], scnt[3];
@@ -240,14 +239,14 @@ __global__ void __launch_bounds__(GEOM_THREADS) mark_kernel(const Lattice L, con
             // bit; the slot's older bits are a subset of prev's (they only
             // accumulate)
             atomicOr(&cur->status, prev->status | ((ovf || mesh_ovf || !sweep_ok) ? ST_BAND_OVERFLOW : 0));
-            if (sweep_ahead(G)) store_sweep(L, G, cur);
         }
     }
     __syncthreads();
+    // (beside the other threads' marks)
+    if (blockIdx.x == 0 && threadIdx.x == 0 && sweep_ahead(G)) store_sweep(L, G, cur);
     const int cap = G.cap[0] * G.cap[1] * G.cap[2];
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= cap) return;
-    for (int c = 0; c < 6; ++c) bforce[(size_t)k * 6 + c] = 0.0;
     int x, y, z;
     if (!band_node(L, G, slo, scnt, k, x, y, z)) return;
     const int n = x + L.nx * (y + L.ny * z);
@@ -278,39 +277,63 @@ __global__ void __launch_bounds__(GEOM_THREADS) classify_kernel(const Lattice L,
 {
     const int cap = G.cap[0] * G.cap[1] * G.cap[2];
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
     int links = 0;
-    int x, y, z;
+    int x, y, z, n = 0;
+    uint32_t m = 0;
+    bool uncovered = false;
     const int lo[3] = {cur->band_lo[0], cur->band_lo[1], cur->band_lo[2]};
     const int cnt[3] = {cur->band_n[0], cur->band_n[1], cur->band_n[2]};
     if (k < cap && band_node(L, G, lo, cnt, k, x, y, z)) {
-        const int n = x + L.nx * (y + L.ny * z);
+        n = x + L.nx * (y + L.ny * z);
         const uint8_t f = flags[n];
         if (!(f & FL_SOLID)) {
             // all 26 neighbour marks are read before any write of this kernel
             // can matter: writes only add BOUNDARY, readers test only SOLID
-            uint32_t m = 0;
+            if (x > 0 && y > 0 && z > 0 && x < L.nx - 1 && y < L.ny - 1 && z < L.nz - 1) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                if (i == 13) continue;
-                const int s = pull_source(L, x, y, z, cx_of(i), cy_of(i), cz_of(i));
-                if (s >= 0 && (flags[s] & FL_SOLID)) m |= 1u << i;
+                for (int i = 0; i < Q; ++i)
+                    if (i != 13 && (flags[n - cx_of(i) - L.nx * (cy_of(i) + L.ny * cz_of(i))] & FL_SOLID)) m |= 1u << i;
+            } else {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    if (i == 13) continue;
+                    const int s = pull_source(L, x, y, z, cx_of(i), cy_of(i), cz_of(i));
+                    if (s >= 0 && (flags[s] & FL_SOLID)) m |= 1u << i;
+                }
             }
             if (m) {
                 flags[n] = f | FL_BOUNDARY;
                 links = __popc(m);
-                const int slot = atomicAdd(&cur->n_boundary, 1);
-                if (slot < G.cap_boundary) { blist[slot] = n; bpos[slot] = k; }
-                else atomicOr(&cur->status, ST_BAND_OVERFLOW);
             }
-            if (f & FL_UNCOVERED) {
-                const int slot = atomicAdd(&cur->n_uncovered, 1);
-                if (slot < G.cap_uncovered) { ulist[slot] = n; upos[slot] = k; }
-                else atomicOr(&cur->status, ST_BAND_OVERFLOW);
-            }
+            uncovered = f & FL_UNCOVERED;
         }
     }
+    // one atomic per warp and list (one per node queued up behind each other:
+    // a sphere of 16 nodes has 600 boundary nodes on one counter)
+    const uint32_t mb = __ballot_sync(0xffffffffu, m != 0), mu = __ballot_sync(0xffffffffu, uncovered);
+    const uint32_t below = (1u << lane) - 1u;
+    if (mb) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&cur->n_boundary, __popc(mb));
+        const int slot = __shfl_sync(0xffffffffu, base, 0) + __popc(mb & below);
+        if (m) {
+            if (slot < G.cap_boundary) { blist[slot] = n; bpos[slot] = k; }
+            else atomicOr(&cur->status, ST_BAND_OVERFLOW);
+        }
+    }
+    if (mu) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&cur->n_uncovered, __popc(mu));
+        const int slot = __shfl_sync(0xffffffffu, base, 0) + __popc(mu & below);
+        if (uncovered) {
+            if (slot < G.cap_uncovered) { ulist[slot] = n; upos[slot] = k; }
+            else atomicOr(&cur->status, ST_BAND_OVERFLOW);
+        }
+    }
+    if (!mb) return;
     for (int o = 16; o > 0; o >>= 1) links += __shfl_down_sync(0xffffffffu, links, o);
-    if ((threadIdx.x & 31) == 0 && links) atomicAdd(&cur->n_links, links);
+    if (lane == 0) atomicAdd(&cur->n_links, links);
 }
 
 // initial marks: SOLID inside the body at X over the whole box
@@ -325,7 +348,11 @@ __global__ void mark_initial_kernel(const Lattice L, const GeomParams G, const d
 }
 
 // ----------------------------------------------------------------- forces
-__global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const GeomParams G, DevBody *__restrict__ cur,
+// (bforce holds a value at the band positions of boundary nodes only: the
+// marks say which, one byte a node in place of clearing and reading 48)
+__global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, const GeomParams G,
+                                                              DevBody *__restrict__ cur,
+                                                              const uint8_t *__restrict__ flags,
                                                               const double *__restrict__ bforce,
                                                               double *__restrict__ partials,
                                                               unsigned *__restrict__ ticket)
@@ -335,8 +362,13 @@ __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const GeomParams G
     const int beg = blockIdx.x * chunk;
     const int end = min(cap, beg + chunk);
     double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int s = beg + threadIdx.x; s < end; s += blockDim.x)
+    const int lo[3] = {cur->band_lo[0], cur->band_lo[1], cur->band_lo[2]};
+    const int cnt[3] = {cur->band_n[0], cur->band_n[1], cur->band_n[2]};
+    for (int s = beg + threadIdx.x; s < end; s += blockDim.x) {
+        int x, y, z;
+        if (!band_node(L, G, lo, cnt, s, x, y, z) || !(flags[x + L.nx * (y + L.ny * z)] & FL_BOUNDARY)) continue;
         for (int c = 0; c < 6; ++c) acc[c] += bforce[(size_t)s * 6 + c];
+    }
     __shared__ double sm[FORCE_THREADS / 32][6];
     __shared__ bool last;
     for (int c = 0; c < 6; ++c) {
@@ -671,7 +703,7 @@ cudaError_t launch_geometry(const Lattice &L, const GeomParams &G, Scratch &S, i
         if (G.com_frame && (e = launch_mesh_body(L, G, S, prev, true, s, nlaunch)) != cudaSuccess) return e;
         if ((e = launch_mesh_prepare(L, G, S, prev, true, s, nlaunch)) != cudaSuccess) return e;
     }
-    mark_kernel<<<nb, GEOM_THREADS, 0, s>>>(L, G, bp, bc, flags, S.bforce);
+    mark_kernel<<<nb, GEOM_THREADS, 0, s>>>(L, G, bp, bc, flags);
     classify_kernel<<<nb, GEOM_THREADS, 0, s>>>(L, G, bc, flags, S.blist, S.bpos, S.ulist, S.upos);
     *nlaunch += 2;
     return cudaGetLastError();
@@ -685,9 +717,10 @@ cudaError_t launch_mark_initial(const Lattice &L, const GeomParams &G, const dou
     return cudaGetLastError();
 }
 
-cudaError_t launch_forces(const GeomParams &G, Scratch &S, int cur, cudaStream_t s, int *nlaunch)
+cudaError_t launch_forces(const Lattice &L, const GeomParams &G, Scratch &S, int cur, const uint8_t *flags,
+                          cudaStream_t s, int *nlaunch)
 {
-    force_kernel<<<S.n_partials, FORCE_THREADS, 0, s>>>(G, S.body + cur, S.bforce, S.partials, S.ticket);
+    force_kernel<<<S.n_partials, FORCE_THREADS, 0, s>>>(L, G, S.body + cur, flags, S.bforce, S.partials, S.ticket);
     *nlaunch += 1;
     return cudaGetLastError();
 }

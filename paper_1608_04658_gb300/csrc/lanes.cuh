@@ -20,6 +20,59 @@ __device__ __forceinline__ R wsum(R v)
     return __shfl_sync(FULL, v, 0);
 }
 
+// Sums of N values over the warp, broadcast to every lane.  At each of the
+// first steps of the butterfly a lane hands on half of its values and keeps
+// the other half, so that N values take about N + 3 exchanges and N
+// broadcasts where one tree each takes 6 N (6 values: 8 + 6 against 36).  The
+// partners of every addition are those of wsum's tree, so each sum has its bits.
+// wsum_scatter6 leaves value k in lane wsum_owner6(k) and the three after it.
+template <typename R>
+__device__ __forceinline__ R wexchange(R keep_lo, R keep_hi, int lane, int o)
+{
+    const bool hi = lane & o;
+    const R keep = hi ? keep_hi : keep_lo, send = hi ? keep_lo : keep_hi;
+    return keep + __shfl_xor_sync(FULL, send, o);
+}
+template <typename R>
+__device__ __forceinline__ R wsum_scatter6(const R v[6], int lane)
+{
+    const R a0 = wexchange(v[0], v[3], lane, 16), a1 = wexchange(v[1], v[4], lane, 16),
+            a2 = wexchange(v[2], v[5], lane, 16);
+    const R b0 = wexchange(a0, a2, lane, 8), b1 = wexchange(a1, R(0), lane, 8);
+    R c = wexchange(b0, b1, lane, 4);
+    c += __shfl_xor_sync(FULL, c, 2);
+    return c + __shfl_xor_sync(FULL, c, 1);
+}
+// the first lane that holds value k of wsum_scatter6
+__host__ __device__ constexpr int wsum_owner6(int k) { return (k >= 3 ? 16 : 0) + (k % 3 == 2 ? 8 : 0) + (k % 3 == 1 ? 4 : 0); }
+template <typename R>
+__device__ __forceinline__ void wsum6(R v[6], int lane)
+{
+    const R c = wsum_scatter6(v, lane);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = __shfl_sync(FULL, c, wsum_owner6(k));
+}
+template <typename R>
+__device__ __forceinline__ void wsum4(R v[4], int lane)
+{
+    const R a0 = wexchange(v[0], v[2], lane, 16), a1 = wexchange(v[1], v[3], lane, 16);
+    R c = wexchange(a0, a1, lane, 8);
+    c += __shfl_xor_sync(FULL, c, 4);
+    c += __shfl_xor_sync(FULL, c, 2);
+    c += __shfl_xor_sync(FULL, c, 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(FULL, c, (k >= 2 ? 16 : 0) + (k & 1 ? 8 : 0));
+}
+template <typename R>
+__device__ __forceinline__ void wsum2(R v[2], int lane)
+{
+    R c = wexchange(v[0], v[1], lane, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) c += __shfl_xor_sync(FULL, c, o);
+    v[0] = __shfl_sync(FULL, c, 0);
+    v[1] = __shfl_sync(FULL, c, 16);
+}
+
 template <typename R>
 __device__ __forceinline__ R pick(const R e[3], int c)
 {
@@ -33,8 +86,10 @@ __device__ R kbc_collide_lanes(R g, int i, R beta, R inv_beta, R rho0, int gamma
     const bool act = i < Q;
     const int cx = act ? cx_of(i) : 0, cy = act ? cy_of(i) : 0, cz = act ? cz_of(i) : 0;
     const R gv = act ? g : R(0);
-    const R drho = wsum(gv);
-    const R jx = wsum(R(cx) * gv), jy = wsum(R(cy) * gv), jz = wsum(R(cz) * gv);
+    const int lane = threadIdx.x & 31;
+    R m4[4] = {gv, R(cx) * gv, R(cy) * gv, R(cz) * gv};
+    wsum4(m4, lane);
+    const R drho = m4[0], jx = m4[1], jy = m4[2], jz = m4[3];
     const R rho = rho0 + drho;
     ok = rho > R(0) && rho < R(1e30);
     const R inv_rho = rcp(rho);
@@ -46,13 +101,16 @@ __device__ R kbc_collide_lanes(R g, int i, R beta, R inv_beta, R rho0, int gamma
     const R E = exy + pick(ez, cz) + exy * pick(ez, cz);
     const R geq = act ? weight<R>(i) * (drho + rho * E) : R(0);
     const R d = gv - geq;
-    const R pxx = wsum(R(cx * cx) * d), pyy = wsum(R(cy * cy) * d), pzz = wsum(R(cz * cz) * d);
-    const R pxy = wsum(R(cx * cy) * d), pxz = wsum(R(cx * cz) * d), pyz = wsum(R(cy * cz) * d);
+    R p6[6] = {R(cx * cx) * d, R(cy * cy) * d, R(cz * cz) * d, R(cx * cy) * d, R(cx * cz) * d, R(cy * cz) * d};
+    wsum6(p6, lane);
+    const R pxx = p6[0], pyy = p6[1], pzz = p6[2], pxy = p6[3], pxz = p6[4], pyz = p6[5];
     const R nxz = pxx - pzz, nyz = pyy - pzz;
     const R ds = act ? shear_part_raw<R>(i, nxz, nyz, pxy, pxz, pyz) : R(0);
     const R dh = d - ds;
     const R ifeq = act ? inv_rho * inv_weight<R>(i) * pick(rx, cx) * pick(ry, cy) * pick(rz, cz) : R(0);
-    const R sh = wsum(ds * dh * ifeq), hh = wsum(dh * dh * ifeq);
+    R s2[2] = {ds * dh * ifeq, dh * dh * ifeq};
+    wsum2(s2, lane);
+    const R sh = s2[0], hh = s2[1];
     R gam = R(2);
     if (gamma_mode != LBM_GAMMA_LBGK && hh > gamma_floor<R>())
         gam = inv_beta - (R(2) - inv_beta) * sh * rcp(hh);
