@@ -1264,7 +1264,7 @@ cudaError_t forward_step(lbm_ctx *ctx, void *fa, void *fb, uint8_t *flags)
             (e = launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, flags, ctx->side)) != cudaSuccess ||
             (e = launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, flags, ctx->side)) !=
                 cudaSuccess ||
-            (ctx->G.free_motion && (e = launch_forces(ctx->L, ctx->G, ctx->S, cur, flags, ctx->side, &nl)) != cudaSuccess) ||
+            (ctx->G.free_motion && (e = launch_forces(ctx->storage, ctx->L, ctx->G, ctx->S, cur, flags, ctx->side, &nl)) != cudaSuccess) ||
             (e = launch_bulk(ctx->storage, ctx->L, fa, fb, flags, status, ctx->side, BULK_BAND, sweep, ctx->G.cap)) !=
                 cudaSuccess ||
             (e = cudaEventRecord(ctx->ev_join, ctx->side)) != cudaSuccess ||
@@ -1287,7 +1287,7 @@ cudaError_t forward_step(lbm_ctx *ctx, void *fa, void *fb, uint8_t *flags)
         if ((e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0)) != cudaSuccess) return e;
         if ((e = launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, flags, ctx->side)) != cudaSuccess)
             return e;
-        if (ctx->G.free_motion && (e = launch_forces(ctx->L, ctx->G, ctx->S, cur, flags, ctx->side, &nl)) != cudaSuccess) return e;
+        if (ctx->G.free_motion && (e = launch_forces(ctx->storage, ctx->L, ctx->G, ctx->S, cur, flags, ctx->side, &nl)) != cudaSuccess) return e;
         if ((e = cudaEventRecord(ctx->ev_join, ctx->side)) != cudaSuccess) return e;
     }
     if ((e = launch_bulk(ctx->storage, ctx->L, fa, fb, fl, status, ctx->stream)) != cudaSuccess) return e;

@@ -476,7 +476,7 @@ lbm_status lbm_set_geometry(lbm_ctx *ctx, const lbm_geometry *g)
     if (body) {
         ok = ctx_alloc(ctx, &S.blist, vol) == cudaSuccess && ctx_alloc(ctx, &S.bpos, vol) == cudaSuccess &&
              ctx_alloc(ctx, &S.ulist, vol) == cudaSuccess && ctx_alloc(ctx, &S.upos, vol) == cudaSuccess &&
-             ctx_alloc(ctx, &S.bforce, vol * 6) == cudaSuccess &&
+             ctx_alloc(ctx, &S.bforce, vol * FORCE_SLOT) == cudaSuccess &&
              ctx_alloc(ctx, &S.partials, (size_t)S.n_partials * 6) == cudaSuccess && ctx_alloc(ctx, &S.ticket, 1) == cudaSuccess;
         if (ok) ok = cudaMemsetAsync(S.ticket, 0, sizeof(unsigned), ctx->stream) == cudaSuccess;
     }
@@ -595,7 +595,7 @@ static cudaError_t sequential_step(lbm_ctx *ctx, void *fa, void *fb, int &cur, i
             (e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0)) != cudaSuccess ||
             (e = launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, ctx->flags, ctx->side)) !=
                 cudaSuccess ||
-            (e = launch_forces(ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches)) != cudaSuccess ||
+            (e = launch_forces(ctx->storage, ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches)) != cudaSuccess ||
             (e = cudaEventRecord(ctx->ev_join, ctx->side)) != cudaSuccess)
             return e;
         launches += 1;
@@ -692,7 +692,7 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
             LBM_CUDA(launch_geometry(ctx->L, ctx->G, ctx->S, prev, ctx->flags, ctx->side, &launches), "geometry");
             LBM_CUDA(launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, ctx->flags, ctx->side), "refill");
             LBM_CUDA(launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, ctx->flags, ctx->side), "boundary");
-            LBM_CUDA(launch_forces(ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches), "forces");
+            LBM_CUDA(launch_forces(ctx->storage, ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches), "forces");
             LBM_CUDA(launch_bulk(ctx->storage, ctx->L, fa, fb, ctx->flags, status, ctx->side, BULK_BAND, sweep,
                                  ctx->G.cap), "bulk band");
             LBM_CUDA(cudaEventRecord(ctx->ev_join, ctx->side), "join");
@@ -780,7 +780,7 @@ lbm_status lbm_step_edges(lbm_ctx *ctx)
         LBM_CUDA(launch_geometry(ctx->L, ctx->G, ctx->S, prev, ctx->flags, ctx->side, &launches), "geometry");
         LBM_CUDA(launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, ctx->flags, ctx->side), "refill");
         LBM_CUDA(launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, ctx->flags, ctx->side), "boundary");
-        LBM_CUDA(launch_forces(ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches), "forces");
+        LBM_CUDA(launch_forces(ctx->storage, ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches), "forces");
         LBM_CUDA(launch_bulk(ctx->storage, ctx->L, fa, fb, ctx->flags, status, ctx->side, BULK_BAND, sweep,
                              ctx->G.cap), "bulk band");
         LBM_CUDA(cudaEventRecord(ctx->ev_join, ctx->side), "join");

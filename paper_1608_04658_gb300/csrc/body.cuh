@@ -85,7 +85,26 @@ struct DevBody {
     int sweep[6];
 };
 
-constexpr int FORCE_BLOCKS = 128;   // blocks (and partial sums) of the force reduction
+// What the boundary kernel leaves of a boundary node's links at its band
+// position (FORCE_SLOT doubles each): the sums of -c (f_out + f_in) + u_w (f_in
+// - f_out) without the rest part, of -q (f_in - f_out) (c x u_w), and the
+// packed integer sums of 216 W c.  With o the node's offset from the reference
+// point, F = sum - 2 rho0 k/216 and M = o x F + h (the wall point is o - q c).
+constexpr int FORCE_SLOT = 7;
+template <typename R> struct ForceSlot;
+template <> struct ForceSlot<double> {
+    double v[6];
+    int k;
+};
+template <> struct ForceSlot<float> {
+    float hi[3], lo[3], h[3];
+    int k;
+};
+__host__ __device__ constexpr int weight216(int i) { return nonzero_of(i) == 0 ? 64 : nonzero_of(i) == 1 ? 16 : nonzero_of(i) == 2 ? 4 : 1; }
+// |k| <= 36 each
+__host__ __device__ constexpr int pack_k(int a, int b, int c) { return (a + 128) | (b + 128) << 8 | (c + 128) << 16; }
+__host__ __device__ constexpr int unpack_k(int k, int a) { return (k >> (8 * a) & 255) - 128; }
+constexpr int FORCE_BLOCKS = 608;   // most blocks (and partial sums) of the force reduction
 
 // scratch owned by the library for the boundary path
 struct Scratch {
@@ -94,7 +113,7 @@ struct Scratch {
     int *bpos;           // [cap_boundary] band position of each boundary node
     int *ulist;          // [cap_uncovered] node index of each uncovered node
     int *upos;           // [cap_uncovered] band position of each uncovered node
-    double *bforce;      // [band capacity * 6] force and torque per band position
+    double *bforce;      // [band capacity * FORCE_SLOT] the links' sums per band position (ForceSlot)
     double *partials;    // [n_partials * 6]
     unsigned *ticket;    // last-block counter of the force reduction
     int n_partials;
@@ -115,7 +134,7 @@ cudaError_t launch_refill(int storage, const Lattice &L, const GeomParams &G, Sc
                           void *fa, const uint8_t *flags, cudaStream_t s);
 cudaError_t launch_boundary(int storage, const Lattice &L, const GeomParams &G, Scratch &S, int cur,
                             const void *fa, void *fb, const uint8_t *flags, cudaStream_t s);
-cudaError_t launch_forces(const Lattice &L, const GeomParams &G, Scratch &S, int cur, const uint8_t *flags,
+cudaError_t launch_forces(int storage, const Lattice &L, const GeomParams &G, Scratch &S, int cur, const uint8_t *flags,
                           cudaStream_t s, int *nlaunch);
 cudaError_t launch_sweep_init(const Lattice &L, const GeomParams &G, Scratch &S, int cur, cudaStream_t s);
 struct Force6 {

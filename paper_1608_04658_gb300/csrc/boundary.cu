@@ -22,6 +22,7 @@
 //   velocity (the swimmer's material velocity at the node's arc position),
 //   gradient with the wall velocity at the centre.
 #include "lanes.cuh"
+#include "pair32.cuh"
 
 namespace lbm {
 
@@ -32,6 +33,80 @@ namespace lbm {
 #ifndef LBM_LIST_MIN_BLOCKS
 #define LBM_LIST_MIN_BLOCKS 7
 #endif
+
+// A boundary node's sums over its links into its slot (see ForceSlot).  FP32
+// and 16-bit storage: sums of -c (f_out + f_in) + u_w (f_in - f_out) without
+// W rho0 as pairs hi + lo of FP32 numbers, error-free but for 2^-48 of values a
+// hundredth of f; W rho0 as the integer sum of 216 W c.  FP64 arithmetic here
+// runs with a fifth of the lanes at work (the missing links of one node) on a
+// pipe of two lanes a clock and SM: it took the larger part of this kernel's
+// time (airfoil 225 us with it).  The force kernel does it for 32 nodes a warp.
+template <typename R>
+__device__ __forceinline__ void node_force(double *__restrict__ slot, int lane, bool link, int cx, int cy, int cz,
+                                           int i, R fbb, R gi, double q, const double uw[3]);
+template <>
+__device__ __forceinline__ void node_force<double>(double *__restrict__ slot, int lane, bool link, int cx, int cy,
+                                                   int cz, int i, double fbb, double gi, double q, const double uw[3])
+{
+    // force without W rho0, and -sum q (f_in - f_out) (c x u_w)
+    double v[6] = {0, 0, 0, 0, 0, 0};
+    if (link) {
+        const double sum = fbb + gi, dif = gi - fbb, h = -q * dif;
+        const int c[3] = {cx, cy, cz};
+        for (int a = 0; a < 3; ++a) {
+            v[a] = fma(uw[a], dif, c[a] == 0 ? 0.0 : (c[a] > 0 ? -sum : sum));
+            const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
+            v[3 + a] = h * (c[b1] * uw[b2] - c[b2] * uw[b1]);
+        }
+    }
+    const double s = wsum_scatter6(v, lane);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (lane == wsum_owner6(k)) reinterpret_cast<ForceSlot<double> *>(slot)->v[k] = s;
+    const int w = link ? weight216(i) : 0;
+    const int k0 = __reduce_add_sync(FULL, w * cx), k1 = __reduce_add_sync(FULL, w * cy),
+              k2 = __reduce_add_sync(FULL, w * cz);
+    if (lane == 0) reinterpret_cast<ForceSlot<double> *>(slot)->k = pack_k(k0, k1, k2);
+}
+template <>
+__device__ __forceinline__ void node_force<float>(double *__restrict__ slot, int lane, bool link, int cx, int cy,
+                                                  int cz, int i, float fbb, float gi, double q, const double uw[3])
+{
+    Pair32 F[3] = {};
+    float H[3] = {0.f, 0.f, 0.f};
+    if (link) {
+        const Pair32 sum = two_sum(fbb, gi), dif = two_sum(gi, -fbb);
+        const int c[3] = {cx, cy, cz};
+        float u[3];
+        for (int a = 0; a < 3; ++a) {
+            u[a] = (float)uw[a];
+            const Pair32 p = Pair32{u[a], (float)(uw[a] - (double)u[a])} * dif;
+            F[a] = c[a] == 0 ? p : (c[a] > 0 ? p - sum : p + sum);
+        }
+        const float h = -(float)q * dif.hi;
+        for (int a = 0; a < 3; ++a) {
+            const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
+            H[a] = h * (c[b1] * u[b2] - c[b2] * u[b1]);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const Pair32 t = {__shfl_xor_sync(FULL, F[a].hi, o), __shfl_xor_sync(FULL, F[a].lo, o)};
+            F[a] = F[a] + t;
+            H[a] += __shfl_xor_sync(FULL, H[a], o);
+        }
+    const int w = link ? weight216(i) : 0;
+    const int k0 = __reduce_add_sync(FULL, w * cx), k1 = __reduce_add_sync(FULL, w * cy),
+              k2 = __reduce_add_sync(FULL, w * cz);
+    if (lane < 3) {
+        ForceSlot<float> *p = reinterpret_cast<ForceSlot<float> *>(slot);
+        p->hi[lane] = lane == 0 ? F[0].hi : (lane == 1 ? F[1].hi : F[2].hi);
+        p->lo[lane] = lane == 0 ? F[0].lo : (lane == 1 ? F[1].lo : F[2].lo);
+        p->h[lane] = lane == 0 ? H[0] : (lane == 1 ? H[1] : H[2]);
+        if (lane == 0) p->k = pack_k(k0, k1, k2);
+    }
+}
 
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_kernel(
@@ -130,32 +205,13 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
         R gi = Fi;
         if (miss) gi = grad_shifted<R>(i, rho_t, rho0, u_t, Qt);
 
-        // momentum exchange on missing links (FP64): the fluid hands the body
-        // (c_opp - u_w) f'_opp(x_b, t) and gets back (c_i - u_w) F_i(x_b, t+1):
-        // -c_i (f_out + f_in) + u_w (f_in - f_out), in which W rho0 leaves the
-        // difference and c_i is a sign
-        double dF[6] = {0, 0, 0, 0, 0, 0};
-        if (miss) {
-            const double fo = (double)fbb, fi = (double)gi;
-            const double sum = (fo + fi) + 2.0 * weight<double>(i) * L.rho0, dif = fi - fo;
-            const int ci[3] = {cx, cy, cz};
-            for (int a = 0; a < 3; ++a) dF[a] = fma(uw[a], dif, ci[a] == 0 ? 0.0 : (ci[a] > 0 ? -sum : sum));
-            const double c[3] = {(double)cx, (double)cy, (double)cz};
-            double r[3];
-            r[0] = body_offset(L, G, b, 0, x) - q * c[0];
-            r[1] = body_offset(L, G, b, 1, y) - q * c[1];
-            r[2] = body_offset(L, G, b, 2, z) - q * c[2];
-            dF[3] = r[1] * dF[2] - r[2] * dF[1];
-            dF[4] = r[2] * dF[0] - r[0] * dF[2];
-            dF[5] = r[0] * dF[1] - r[1] * dF[0];
-        }
+        // momentum exchange on missing links: the fluid hands the body
+        // (c_opp - u_w) f'_opp(x_b, t) and gets back (c_i - u_w) F_i(x_b, t+1),
+        // together -c_i (f_out + f_in) + u_w (f_in - f_out); the node's sums go
+        // into its band slot, which the force kernel turns into force and torque
         // a slab's links count where it owns the fluid node
         const bool own = z >= G.own_lo && z < G.own_hi;
-        const double fsum = wsum_scatter6(dF, lane);
-        const size_t pos = (size_t)bpos[slot] * 6;
-#pragma unroll
-        for (int k = 0; k < 6; ++k)
-            if (lane == wsum_owner6(k)) bforce[pos + k] = own ? fsum : 0.0;
+        node_force<R>(bforce + (size_t)bpos[slot] * FORCE_SLOT, lane, own && miss, cx, cy, cz, i, fbb, gi, q, uw);
 
         bool ok;
         const R out = kbc_collide_lanes<R>(gi, i, (R)L.beta, (R)L.inv_beta, rho0, L.gamma_mode, ok);
@@ -225,12 +281,13 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) refill_kerne
 #ifndef LBM_LIST_BLOCKS
 #define LBM_LIST_BLOCKS 304
 #endif
-// The swimmer's boundary nodes each carry a triangle search, so its
-// boundary kernel is the long part of the body's launch chain:
-// LBM_MESH_LIST_BLOCKS gives it more blocks (608 took the 256x128x128
-// swimmer's step from 0.359 to 0.256 ms).
-#ifndef LBM_MESH_LIST_BLOCKS
-#define LBM_MESH_LIST_BLOCKS 608
+// The links of the swimmer (a triangle search) and of the airfoil (a bisection)
+// make their boundary kernel the long part of the body's launch chain:
+// LBM_LINK_LIST_BLOCKS gives it more blocks (608 took the 256x128x128
+// swimmer's step from 0.359 to 0.256 ms and the two-level airfoil's coarse
+// step from 1.13 to 1.05 ms; 1064 measured 1.07).
+#ifndef LBM_LINK_LIST_BLOCKS
+#define LBM_LINK_LIST_BLOCKS 608
 #endif
 static int list_blocks(int cap, int max_blocks = LBM_LIST_BLOCKS)
 {
@@ -243,7 +300,7 @@ cudaError_t launch_boundary(int storage, const Lattice &L, const GeomParams &G, 
 {
     return dispatch_storage(storage, [&](auto tag) {
         using T = std::remove_pointer_t<decltype(tag)>;
-        const int nb = list_blocks(G.cap_boundary, G.kind == LBM_BODY_MESH ? LBM_MESH_LIST_BLOCKS : LBM_LIST_BLOCKS);
+        const int nb = list_blocks(G.cap_boundary, G.kind == LBM_BODY_MESH || G.kind == LBM_BODY_AIRFOIL ? LBM_LINK_LIST_BLOCKS : LBM_LIST_BLOCKS);
         boundary_kernel<T><<<nb, BWARPS * 32, 0, s>>>(L, G, S.body + cur, S.blist, S.bpos, S.bforce, (const T *)fa,
                                                       (T *)fb, flags);
         return cudaGetLastError();

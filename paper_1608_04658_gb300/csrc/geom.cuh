@@ -349,17 +349,21 @@ __device__ void mesh_links_warp(const GeomParams &G, const DevBody *b, int x, in
             hitout.tri = bt;
             hitout.u = bu;
             hitout.v = bv;
-            if (bt < 0) {
-                q = 0.5;
-                mesh_material_velocity(G, b, (double)x - 0.5 * c[0], (double)y - 0.5 * c[1], uw);
-            } else {
-                q = best;
-                const int t0 = G.mesh_tris[3 * bt], t1 = G.mesh_tris[3 * bt + 1], t2 = G.mesh_tris[3 * bt + 2];
-                for (int a = 0; a < 3; ++a)
-                    uw[a] = (1.0 - bu - bv) * G.mesh_vel[3 * t0 + a] + bu * G.mesh_vel[3 * t1 + a] +
-                            bv * G.mesh_vel[3 * t2 + a];
-            }
+            q = best;
         }
+    }
+    // the wall velocities of all links at once (FP64: one pass of the pipe for
+    // the node, not one for each link)
+    if (!((mask >> lane) & 1u)) return;
+    if (hitout.tri < 0) {
+        q = 0.5;
+        mesh_material_velocity(G, b, (double)x - 0.5 * cx_of(lane), (double)y - 0.5 * cy_of(lane), uw);
+    } else {
+        const int bt = hitout.tri;
+        const int t0 = G.mesh_tris[3 * bt], t1 = G.mesh_tris[3 * bt + 1], t2 = G.mesh_tris[3 * bt + 2];
+        for (int a = 0; a < 3; ++a)
+            uw[a] = (1.0 - hitout.u - hitout.v) * G.mesh_vel[3 * t0 + a] + hitout.u * G.mesh_vel[3 * t1 + a] +
+                    hitout.v * G.mesh_vel[3 * t2 + a];
     }
 }
 
@@ -395,7 +399,7 @@ __device__ __forceinline__ double link_airfoil_f(const GeomParams &G, const DevB
         if (inside_airfoil_f(G, xi0 + mid * dxi, eta0 + mid * deta)) hi = mid;
         else lo = mid;
     }
-    return 0.5 * ((double)lo + (double)hi);
+    return (double)lo + 0x1p-25;  // the middle of [lo, lo + 2^-24]
 }
 
 // Pull source x - c under the box rules; node index, or -1 when a wall or

@@ -14,7 +14,9 @@
 //             the band in a fixed assignment, then the last block to finish
 //             adds the partials with a fixed shuffle tree.  The result does not
 //             depend on list order or block timing.
-#include "geom.cuh"
+#include <algorithm>
+
+#include "lanes.cuh"
 
 namespace lbm {
 
@@ -350,6 +352,7 @@ __global__ void mark_initial_kernel(const Lattice L, const GeomParams G, const d
 // ----------------------------------------------------------------- forces
 // (bforce holds a value at the band positions of boundary nodes only: the
 // marks say which, one byte a node in place of clearing and reading 48)
+template <typename R>
 __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, const GeomParams G,
                                                               DevBody *__restrict__ cur,
                                                               const uint8_t *__restrict__ flags,
@@ -362,19 +365,61 @@ __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, c
     const int beg = blockIdx.x * chunk;
     const int end = min(cap, beg + chunk);
     double acc[6] = {0, 0, 0, 0, 0, 0};
+    bool used = false;
     const int lo[3] = {cur->band_lo[0], cur->band_lo[1], cur->band_lo[2]};
     const int cnt[3] = {cur->band_n[0], cur->band_n[1], cur->band_n[2]};
-    for (int s = beg + threadIdx.x; s < end; s += blockDim.x) {
+    // The boundary nodes of FORCE_THREADS positions at a time are first packed
+    // (a fifteenth of a band's nodes: unpacked, nearly every warp would go through
+    // the FP64 arithmetic for one or two of its lanes), in band order
+    __shared__ int spos[FORCE_THREADS], scount[FORCE_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int s0 = beg; s0 < end; s0 += FORCE_THREADS) {
+        const int s = s0 + threadIdx.x;
         int x, y, z;
-        if (!band_node(L, G, lo, cnt, s, x, y, z) || !(flags[x + L.nx * (y + L.ny * z)] & FL_BOUNDARY)) continue;
-        for (int c = 0; c < 6; ++c) acc[c] += bforce[(size_t)s * 6 + c];
+        const bool at = s < end && band_node(L, G, lo, cnt, s, x, y, z) &&
+                        (flags[x + L.nx * (y + L.ny * z)] & FL_BOUNDARY);
+        const unsigned mask = __ballot_sync(0xffffffffu, at);
+        if (lane == 0) scount[warp] = __popc(mask);
+        __syncthreads();
+        int base = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < FORCE_THREADS / 32; ++w) {
+            base += w < warp ? scount[w] : 0;
+            total += scount[w];
+        }
+        if (at) spos[base + __popc(mask & ((1u << lane) - 1u))] = s;
+        __syncthreads();
+        if ((int)threadIdx.x >= total) continue;
+        used = true;
+        const int k = spos[threadIdx.x];
+        band_node(L, G, lo, cnt, k, x, y, z);
+        const ForceSlot<R> *p = reinterpret_cast<const ForceSlot<R> *>(bforce + (size_t)k * FORCE_SLOT);
+        double F[3], h[3];
+        const int kk = p->k;
+        for (int a = 0; a < 3; ++a) {
+            if constexpr (sizeof(R) == 8) {
+                F[a] = p->v[a];
+                h[a] = p->v[3 + a];
+            } else {
+                F[a] = (double)p->hi[a] + (double)p->lo[a];
+                h[a] = (double)p->h[a];
+            }
+            F[a] -= (L.rho0 / 108.0) * unpack_k(kk, a);
+        }
+        const double o[3] = {body_offset(L, G, cur, 0, x), body_offset(L, G, cur, 1, y), body_offset(L, G, cur, 2, z)};
+        for (int a = 0; a < 3; ++a) {
+            const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
+            acc[a] += F[a];
+            acc[3 + a] += o[b1] * F[b2] - o[b2] * F[b1] + h[a];
+        }
     }
     __shared__ double sm[FORCE_THREADS / 32][6];
     __shared__ bool last;
-    for (int c = 0; c < 6; ++c) {
-        double v = acc[c];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5][c] = v;
+    {
+        const double v = __any_sync(0xffffffffu, used) ? wsum_scatter6(acc, lane) : 0.0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (lane == wsum_owner6(k)) sm[warp][k] = v;
     }
     __syncthreads();
     if (threadIdx.x < 6) {
@@ -389,7 +434,7 @@ __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, c
     if (!last) return;
     __threadfence();
     // last block: component c = warp c, lanes take partials lane, lane + 32, ...
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int w = warp;
     if (w < 6) {
         double v = 0;
         for (int p = lane; p < (int)gridDim.x; p += 32) v += ((volatile double *)partials)[p * 6 + w];
@@ -717,10 +762,15 @@ cudaError_t launch_mark_initial(const Lattice &L, const GeomParams &G, const dou
     return cudaGetLastError();
 }
 
-cudaError_t launch_forces(const Lattice &L, const GeomParams &G, Scratch &S, int cur, const uint8_t *flags,
+cudaError_t launch_forces(int storage, const Lattice &L, const GeomParams &G, Scratch &S, int cur, const uint8_t *flags,
                           cudaStream_t s, int *nlaunch)
 {
-    force_kernel<<<S.n_partials, FORCE_THREADS, 0, s>>>(L, G, S.body + cur, flags, S.bforce, S.partials, S.ticket);
+    auto kernel = storage == LBM_FP64 ? force_kernel<double> : force_kernel<float>;
+    // two packings of FORCE_THREADS positions a block: each costs two barriers
+    // and a round trip to memory (airfoil, 240,000 positions: 128 blocks 28 us)
+    const long long cap = (long long)G.cap[0] * G.cap[1] * G.cap[2];
+    const int nb = (int)std::min<long long>(S.n_partials, (cap + 2 * FORCE_THREADS - 1) / (2 * FORCE_THREADS));
+    kernel<<<nb, FORCE_THREADS, 0, s>>>(L, G, S.body + cur, flags, S.bforce, S.partials, S.ticket);
     *nlaunch += 1;
     return cudaGetLastError();
 }
