@@ -127,7 +127,7 @@ lbm_status lbm_create(const lbm_params *p, void *f_a, void *f_b, uint8_t *flags,
     lbm_ctx *ctx = new (std::nothrow) lbm_ctx();
     if (!ctx) return LBM_ERR_OOM;
     Lattice &L = ctx->L;
-    L.nx = p->nx; L.ny = p->ny; L.nz = p->nz; L.N = N;
+    L.nx = p->nx; L.ny = p->ny; L.nz = p->nz; L.N = L.n_box = N;
     for (int i = 0; i < Q; ++i) L.plane[i] = (int)(i * N);
     for (int k = 0; k < 6; ++k) L.face[k] = p->face[k];
     L.gamma_mode = p->gamma_mode;
@@ -139,6 +139,7 @@ lbm_status lbm_create(const lbm_params *p, void *f_a, void *f_b, uint8_t *flags,
     L.beta_f = (float)L.beta;
     L.inv_beta_f = (float)L.inv_beta;
     L.rho0_f = (float)L.rho0;
+    L.zero_f = 0.0f;
     for (int i = 0; i < Q; ++i) L.g_face_f[i] = (float)L.g_face[i];
     ctx->storage = p->storage;
     ctx->elem = es;
@@ -1129,6 +1130,7 @@ lbm_status lbm_set_slab(lbm_ctx *ctx, int zoff, int zper, int own_lo, int own_hi
     ctx->slab_zper = zper;
     ctx->slab_own_lo = own_lo;
     ctx->slab_own_hi = own_hi;
+    ctx->L.n_box = (long long)L.nx * L.ny * zper;
     return LBM_OK;
 }
 

@@ -18,11 +18,14 @@ namespace lbm {
 // one node: V = float
 struct F1 {
     using V = float;
-    static __device__ __forceinline__ V c(float s) { return s; }
+    using R = float;
+    static __device__ __forceinline__ V c(double s) { return (float)s; }
+    static __device__ __forceinline__ V bc(float s) { return s; }
     static __device__ __forceinline__ V add(V a, V b) { return __fadd_rn(a, b); }
     static __device__ __forceinline__ V sub(V a, V b) { return __fadd_rn(a, -b); }
     static __device__ __forceinline__ V mul(V a, V b) { return __fmul_rn(a, b); }
     static __device__ __forceinline__ V fma(V a, V b, V d) { return __fmaf_rn(a, b, d); }
+    static __device__ __forceinline__ V fnma(V a, V b, V d) { return __fmaf_rn(-a, b, d); }
     static __device__ __forceinline__ V neg(V a) { return -a; }
     static __device__ __forceinline__ V rcp(V a) { return rcp_fast(a); }
     static __device__ __forceinline__ V sqrt(V a) { return sqrt_fast(a); }
@@ -33,11 +36,14 @@ struct F1 {
 // two nodes: V = float2, lane x the first node, lane y the second
 struct F2 {
     using V = float2;
-    static __device__ __forceinline__ V c(float s) { return make_float2(s, s); }
+    using R = float;
+    static __device__ __forceinline__ V c(double s) { return make_float2((float)s, (float)s); }
+    static __device__ __forceinline__ V bc(float s) { return make_float2(s, s); }
     static __device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
     static __device__ __forceinline__ V sub(V a, V b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
     static __device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
     static __device__ __forceinline__ V fma(V a, V b, V d) { return __ffma2_rn(a, b, d); }
+    static __device__ __forceinline__ V fnma(V a, V b, V d) { return __ffma2_rn(make_float2(-a.x, -a.y), b, d); }
     static __device__ __forceinline__ V neg(V a) { return make_float2(-a.x, -a.y); }
     static __device__ __forceinline__ V rcp(V a) { return make_float2(rcp_fast(a.x), rcp_fast(a.y)); }
     static __device__ __forceinline__ V sqrt(V a) { return make_float2(sqrt_fast(a.x), sqrt_fast(a.y)); }

@@ -76,6 +76,7 @@ template <> struct Codec<__nv_bfloat16> {
 struct Lattice {
     int nx, ny, nz;
     long long N;
+    long long n_box;    // N, or the nodes of the whole box a slab belongs to
     int plane[27];      // i * N: offset of population plane i (27 N < 2^31)
     int face[6];
     int gamma_mode;
@@ -88,6 +89,7 @@ struct Lattice {
     // bulk kernels (no FP64 conversion on the device)
     float beta_f, inv_beta_f, rho0_f;
     float g_face_f[27];
+    float zero_f;       // 0, not known to the compiler (see kbc_collide_v)
 };
 
 // Which nodes one bulk launch updates.  ALL: every node (those flagged SOLID

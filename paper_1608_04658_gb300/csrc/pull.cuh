@@ -3,7 +3,7 @@
 // its adjoint.
 #pragma once
 
-#include "kbcv.cuh"
+#include "kbcm.cuh"
 
 namespace lbm {
 
@@ -108,52 +108,30 @@ __device__ __forceinline__ void gather_global(const Lattice &L, const S *__restr
     }
 }
 
-// The pulls of one node, as gather_global, written into lane H (0: x, 1: y)
-// of the float2 populations of a node pair (the pair's node at an x face).
-template <typename S, int H>
-__device__ __forceinline__ void gather_node_lane(const Lattice &L, const S *__restrict__ fa, int x, int y, int z,
-                                                 int n, float2 g[Q])
-{
-    int ox[3], oy[3], oz[3], kx[3], ky[3], kz[3];
-    axis_off(x, L.nx, 1, L.face[0], L.face[1], ox, kx);
-    axis_off(y, L.ny, L.nx, L.face[2], L.face[3], oy, ky);
-    axis_off(z, L.nz, L.nx * L.ny, L.face[4], L.face[5], oz, kz);
-    const S *p = fa + n;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int k = max(kx[cx_of(i) + 1], max(ky[cy_of(i) + 1], kz[cz_of(i) + 1]));
-        const float v = k == 2 ? (float)Codec<S>::load(p + L.plane[26 - i])
-                      : k == 1 ? L.g_face_f[i]
-                               : (float)Codec<S>::load(p + (L.plane[i] + ox[cx_of(i) + 1] + oy[cy_of(i) + 1] +
-                                                            oz[cz_of(i) + 1]));
-        if (H) g[i].y = v;
-        else g[i].x = v;
-    }
-}
-
 // Storage word of two consecutive nodes along x: FP32 as float2 (8 bytes),
-// 16-bit as a 4-byte pair; cross(a, b) is the pair (second node of a, first
-// node of b).  The word address is even in nodes (n even, every plane and
-// row offset even when nx is even), so these are aligned vector accesses.
+// 16-bit as a 4-byte pair; cross(a, b) gives the values of (second node of a,
+// first node of b), each half converted where it lies.  The word address is
+// even in nodes (n even, every plane and row offset even when nx is even), so
+// these are aligned vector accesses.
 template <typename S> struct Pair;
 template <> struct Pair<float> {
     using W = float2;
     __device__ static W load(const float *p) { return *reinterpret_cast<const float2 *>(p); }
-    __device__ static W cross(W a, W b) { return make_float2(a.y, b.x); }
+    __device__ static float2 cross(W a, W b) { return make_float2(a.y, b.x); }
     __device__ static float2 unpack(W w) { return w; }
     __device__ static void store(float *p, float2 v) { *reinterpret_cast<float2 *>(p) = v; }
 };
 template <> struct Pair<__half> {
     using W = __half2;
     __device__ static W load(const __half *p) { return *reinterpret_cast<const __half2 *>(p); }
-    __device__ static W cross(W a, W b) { return __halves2half2(__high2half(a), __low2half(b)); }
+    __device__ static float2 cross(W a, W b) { return make_float2(__high2float(a), __low2float(b)); }
     __device__ static float2 unpack(W w) { return __half22float2(w); }
     __device__ static void store(__half *p, float2 v) { *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v.x, v.y); }
 };
 template <> struct Pair<__nv_bfloat16> {
     using W = __nv_bfloat162;
     __device__ static W load(const __nv_bfloat16 *p) { return *reinterpret_cast<const __nv_bfloat162 *>(p); }
-    __device__ static W cross(W a, W b) { return __halves2bfloat162(__high2bfloat16(a), __low2bfloat16(b)); }
+    __device__ static float2 cross(W a, W b) { return make_float2(__high2float(a), __low2float(b)); }
     __device__ static float2 unpack(W w) { return __bfloat1622float2(w); }
     __device__ static void store(__nv_bfloat16 *p, float2 v)
     {
@@ -161,7 +139,7 @@ template <> struct Pair<__nv_bfloat16> {
     }
 };
 
-// Pulls of the node pair (x0, x0 + 1), x0 even, nx even.  Every load of the
+// Pulls of the node pair (x0, x0 + 1), x0 even; nx even, or ODD and x0 + 1 < nx.  Every load of the
 // pair is issued in one pass with addresses chosen by selects (a branch there
 // would hold back the later loads until the earlier ones return).
 //   XPER and YZPER (periodic box): per direction the source word of the pair
@@ -172,10 +150,9 @@ template <> struct Pair<__nv_bfloat16> {
 //   wrapped node (periodic), the node's own opposite population (wall) or the
 //   clamped source (outflow).  y and z faces, uniform over the pair's row,
 //   are applied after the loads: a wall takes the pair's own opposite word
-//   (loaded then), an equilibrium face its value.  A node on an equilibrium x
-//   face, or on an x wall of a row with an equilibrium y or z face, is
-//   gathered again on its own.
-template <typename S, bool XPER, bool YZPER>
+//   (loaded then), an equilibrium face its value (not over an x wall's), and an
+//   equilibrium x face its value in the outer node (not over a y or z wall's).
+template <typename S, bool XPER, bool YZPER, bool ODD>
 __device__ __forceinline__ void gather_pair(const Lattice &L, const S *__restrict__ fa, int x0, int y, int z,
                                             int n0, float2 g[Q])
 {
@@ -192,8 +169,8 @@ __device__ __forceinline__ void gather_pair(const Lattice &L, const S *__restric
             const S *q = p + (L.plane[i] + oy[cy_of(i) + 1] + oz[cz_of(i) + 1]);
             const typename P::W w = P::load(q);
             if (cx == 0) g[i] = P::unpack(w);
-            else if (cx > 0) g[i] = P::unpack(P::cross(P::load(q + xl), w));   // sources x0 - 1, x0
-            else g[i] = P::unpack(P::cross(w, P::load(q + xr)));               // sources x0 + 1, x0 + 2
+            else if (cx > 0) g[i] = P::cross(P::load(q + xl), w);   // sources x0 - 1, x0
+            else g[i] = P::cross(w, P::load(q + xr));               // sources x0 + 1, x0 + 2
         }
     } else {
         // element offsets (from the pair's first node) of the outer node of the
@@ -201,25 +178,26 @@ __device__ __forceinline__ void gather_pair(const Lattice &L, const S *__restric
         // relative to the source word, or the own opposite population when
         // own_l / own_r (a wall)
         int dl = -1, dr = 2;
-        bool own_l = false, own_r = false, again_l = false, again_r = false;
-        const bool eq_yz = !YZPER && ((ky[0] | ky[2] | kz[0] | kz[2]) & 1);
+        bool own_l = false, own_r = false, eq_l = false, eq_r = false;
         if (x0 == 0) {
             const int f = L.face[0];
             dl = f == LBM_FACE_PERIODIC ? L.nx - 1 : 0;  // outflow: the clamped source x0
             own_l = f == LBM_FACE_WALL;
-            again_l = f == LBM_FACE_EQ || (own_l && eq_yz);
+            eq_l = f == LBM_FACE_EQ;
         }
         if (x0 + 2 >= L.nx) {
             const int f = L.face[1];
             dr = f == LBM_FACE_PERIODIC ? 2 - L.nx : 1;  // outflow: the clamped source x0 + 1
             own_r = f == LBM_FACE_WALL;
-            again_r = f == LBM_FACE_EQ || (own_r && eq_yz);
+            eq_r = f == LBM_FACE_EQ;
         }
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int cx = cx_of(i);
             const int src = L.plane[i] + oy[cy_of(i) + 1] + oz[cz_of(i) + 1];
-            const float2 m = P::unpack(P::load(p + src));
+            // (rows of odd length: the two words of a pair are single elements)
+            const float2 m = ODD ? make_float2((float)Codec<S>::load(p + src), (float)Codec<S>::load(p + src + 1))
+                                 : P::unpack(P::load(p + src));
             if (cx == 0) {
                 g[i] = m;
             } else if (cx > 0) {
@@ -234,12 +212,24 @@ __device__ __forceinline__ void gather_pair(const Lattice &L, const S *__restric
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const int k = max(ky[cy_of(i) + 1], kz[cz_of(i) + 1]);
-                if (k == 2) g[i] = P::unpack(P::load(p + L.plane[26 - i]));  // the pair's own bounce-back word
-                else if (k == 1) g[i] = make_float2(L.g_face_f[i], L.g_face_f[i]);
+                if (k == 2) {  // the pair's own bounce-back word
+                    const S *o = p + L.plane[26 - i];
+                    g[i] = ODD ? make_float2((float)Codec<S>::load(o), (float)Codec<S>::load(o + 1)) : P::unpack(P::load(o));
+                }
+                else if (k == 1) {
+                    if (!(cx_of(i) > 0 && own_l)) g[i].x = L.g_face_f[i];
+                    if (!(cx_of(i) < 0 && own_r)) g[i].y = L.g_face_f[i];
+                }
             }
         }
-        if (again_l) gather_node_lane<S, 0>(L, fa, 0, y, z, n0, g);
-        if (again_r) gather_node_lane<S, 1>(L, fa, L.nx - 1, y, z, n0 + 1, g);
+        if (eq_l || eq_r) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                if (cx_of(i) == 0 || (!YZPER && max(ky[cy_of(i) + 1], kz[cz_of(i) + 1]) == 2)) continue;
+                if (cx_of(i) > 0 && eq_l) g[i].x = L.g_face_f[i];
+                if (cx_of(i) < 0 && eq_r) g[i].y = L.g_face_f[i];
+            }
+        }
     }
 }
 
