@@ -410,6 +410,35 @@ __device__ __noinline__ R next_adjoint_rare(const Lattice &L, const GeomParams &
     return next_adjoint<R>(L, G, A, x, y, z, n, i);
 }
 
+// lambda(S^{t+1})(x) of all directions: off the faces that need more, 27 plain
+// loads and the band's extra terms
+template <typename R>
+__device__ __forceinline__ void next_adjoint_all(const Lattice &L, const GeomParams &G, const NextAdj<R> &A, int x,
+                                                 int y, int z, int n, R (&lam)[Q])
+{
+    const size_t N = (size_t)L.N;
+    int ox[3], oy[3], oz[3];
+    bool special = axis_readers(x, L.nx, 1, L.face[0], L.face[1], ox);
+    special |= axis_readers(y, L.ny, L.nx, L.face[2], L.face[3], oy);
+    special |= axis_readers(z, L.nz, L.nx * L.ny, L.face[4], L.face[5], oz);
+    if (A.direct || special || (A.flags && (A.flags[n] & FL_UNCOVERED))) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) lam[i] = next_adjoint_rare<R>(L, G, A, x, y, z, n, i);
+    } else {
+        const R *p = A.lam + n;
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            lam[i] = p[(long long)i * (long long)N + (ox[cx_of(i) + 1] + oy[cy_of(i) + 1] + oz[cz_of(i) + 1])];
+        if (A.ext) {
+            const int k = band_index(L, G, A.band, x, y, z);
+            if (k >= 0) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) lam[i] += (R)A.ext[(size_t)k * Q + i];
+            }
+        }
+    }
+}
+
 // ----------------------------------------------------------------- kernels
 // Nodes fluid at t+1 without missing links: Lam^t(x) = C'(F(x))^T lambda(S^{t+1})(x);
 // solid nodes get Lam^t = 0; boundary nodes are left to the boundary adjoint.
@@ -461,26 +490,7 @@ __global__ void __launch_bounds__(128, LBM_ADJ_MIN_BLOCKS) adjoint_bulk_kernel(c
     }
     if (f1 & FL_BOUNDARY) return;
     R lam[Q];
-    int ox[3], oy[3], oz[3];
-    bool special = axis_readers(x, L.nx, 1, L.face[0], L.face[1], ox);
-    special |= axis_readers(y, L.ny, L.nx, L.face[2], L.face[3], oy);
-    special |= axis_readers(z, L.nz, L.nx * L.ny, L.face[4], L.face[5], oz);
-    if (A.direct || special || (A.flags && (A.flags[n] & FL_UNCOVERED))) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) lam[i] = next_adjoint_rare<R>(L, G, A, x, y, z, n, i);
-    } else {
-        const R *p = A.lam + n;
-#pragma unroll
-        for (int i = 0; i < Q; ++i)
-            lam[i] = p[(long long)i * (long long)N + (ox[cx_of(i) + 1] + oy[cy_of(i) + 1] + oz[cz_of(i) + 1])];
-        if (A.ext) {
-            const int k = band_index(L, G, A.band, x, y, z);
-            if (k >= 0) {
-#pragma unroll
-                for (int i = 0; i < Q; ++i) lam[i] += (R)A.ext[(size_t)k * Q + i];
-            }
-        }
-    }
+    next_adjoint_all<R>(L, G, A, x, y, z, n, lam);
     R g[Q];
     gather_global<S>(L, st, x, y, z, n, g);
     kbc_vjp<R>(g, lam, (R)L.beta, (R)L.inv_beta, (R)L.rho0, L.gamma_mode);
@@ -730,6 +740,7 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
     using R = typename Codec<S>::R;
     __shared__ R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
+    __shared__ LinkScratch s_link[BWARPS];
     __shared__ int s_ok[BWARPS][Q];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     R (*sf)[28] = s_f[w];
@@ -785,7 +796,7 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
         const R fbb = act ? sf[13][26 - (act ? i : 0)] : R(0);
         double q = 0, uw[3] = {0, 0, 0};
         MeshHit hit{-1, 0.0, 0.0};
-        if (G.kind == LBM_BODY_MESH) mesh_links_warp<R>(G, b, x, y, z, mask, lane, q, uw, hit);
+        if (G.kind == LBM_BODY_MESH) mesh_links_warp<R>(G, b, x, y, z, mask, lane, q, uw, hit, s_link[w]);
         else if (miss) link_data<R>(L, G, b, x, y, z, cx, cy, cz, q, uw);
         const R gstat = miss ? fbb : Fi;
         const R dyn = miss ? R(6) * weight<R>(i) * rho0 * (R(cx) * (R)uw[0] + R(cy) * (R)uw[1] + R(cz) * (R)uw[2])
@@ -1159,12 +1170,16 @@ __global__ void __launch_bounds__(256) theta_reduce_kernel(const double *__restr
 // lambda(S^0): the transpose of step 0's pull and band contributions, zero at
 // nodes refilled in step 0
 template <typename R>
-__global__ void lambda0_kernel(const Lattice L, const GeomParams G, const NextAdj<R> A, R *__restrict__ out)
+__global__ void __launch_bounds__(128) lambda0_kernel(const Lattice L, const GeomParams G, const NextAdj<R> A,
+                                                      R *__restrict__ out)
 {
-    const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= L.N) return;
-    const int x = (int)(n % L.nx), y = (int)((n / L.nx) % L.ny), z = (int)(n / ((long long)L.nx * L.ny));
-    for (int i = 0; i < Q; ++i) out[(size_t)i * (size_t)L.N + n] = next_adjoint<R>(L, G, A, x, y, z, (int)n, i);
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+    if (x >= L.nx) return;
+    const int n = x + L.nx * (y + L.ny * z);
+    R lam[Q];
+    next_adjoint_all<R>(L, G, A, x, y, z, n, lam);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) out[(size_t)i * (size_t)L.N + n] = lam[i];
 }
 
 // per-block partial sums of lambda_T . f over nodes fluid at the end
@@ -1631,7 +1646,8 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
         // lambda(S^0) from the last reversed step (step 0)
         if (spec->lambda_0) {
             NextAdj<R> A{lam[p ^ 1], body ? ext[p ^ 1] : nullptr, adjbody + (p ^ 1), body ? wf[p ^ 1] : nullptr, 0};
-            lambda0_kernel<R><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(L, ctx->G, A, (R *)spec->lambda_0);
+            const int bx = L.nx >= 128 ? 128 : ((L.nx + 31) / 32) * 32;
+            lambda0_kernel<R><<<dim3((L.nx + bx - 1) / bx, L.ny, L.nz), bx, 0, s>>>(L, ctx->G, A, (R *)spec->lambda_0);
             ADJ_CUDA(cudaGetLastError(), "lambda0");
         }
     }

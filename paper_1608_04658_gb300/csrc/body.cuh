@@ -11,7 +11,11 @@ namespace lbm {
 constexpr int MESH_COL_CAP = 32;    // crossings kept per band column
 constexpr int MESH_CELL = 2;        // edge of a triangle cell (lattice units)
 constexpr int MESH_CELL_CAP = 384;  // triangles kept per cell
-constexpr int MESH_THREADS = 256;   // block size of the per-vertex and per-triangle mesh kernels
+constexpr int MESH_THREADS = 256;   // block size of the volume sums' kernel (per triangle)
+// Block size of the per-vertex and per-triangle pose kernels: their FP64
+// arithmetic (sines, divisions) is a queue on each SM's two FP64 lanes a clock,
+// so the warps are spread over all SMs, not over 38 to 75 blocks of 256 threads
+constexpr int POSE_THREADS = 32;
 
 struct GeomParams {
     int kind;

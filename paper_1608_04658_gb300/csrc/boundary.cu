@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
     using R = typename Codec<S>::R;
     __shared__ R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
+    __shared__ LinkScratch s_link[BWARPS];
     __shared__ int s_ok[BWARPS][Q];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     R (*sf)[28] = s_f[w];
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
         double q = 0, uw[3] = {0, 0, 0};
         if (G.kind == LBM_BODY_MESH) {
             MeshHit hit{-1, 0.0, 0.0};
-            mesh_links_warp<R>(G, b, x, y, z, mask, lane, q, uw, hit);
+            mesh_links_warp<R>(G, b, x, y, z, mask, lane, q, uw, hit, s_link[w]);
         } else if (miss) {
             link_data<R>(L, G, b, x, y, z, cx, cy, cz, q, uw);
         }

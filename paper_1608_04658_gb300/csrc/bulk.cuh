@@ -208,12 +208,19 @@ cudaError_t launch_bulk_form(const Lattice &L, const S *fa, S *fb, const uint8_t
                              int mode, const int *sweep, const int *cap, int z_lo, int z_n)
 {
     // FP32 and 16-bit storage take the two-node kernel for everything but the
-    // sweep box (every node gets the same bits either way)
+    // sweep box (every node gets the same bits either way).  FP32 rows of odd
+    // length stay with the one-node kernel, whose whole lines suit a launch bound
+    // by memory (147x21x180: 27 us a step, 30 as unaligned pairs; in 16 bits, bound
+    // by arithmetic, 161x97x83 57 against 44), but for the exact stabilizer.
     if constexpr (!std::is_same<S, double>::value) {
-        if (mode != BULK_BAND && L.nx > 1) {
-            const bool odd = L.nx & 1, xper = L.face[0] == LBM_FACE_PERIODIC,
+        constexpr bool odd_pairs = sizeof(S) == 2 || FORM == FORM_MX;
+        const bool odd = L.nx & 1;
+        if (mode != BULK_BAND && L.nx > 1 && (odd_pairs || !odd)) {
+            const bool xper = L.face[0] == LBM_FACE_PERIODIC,
                        yzper = L.face[2] == LBM_FACE_PERIODIC && L.face[4] == LBM_FACE_PERIODIC;
-            auto kernel = odd ? bulk_pair_kernel<S, FORM, false, false, true> : bulk_pair_kernel<S, FORM, false, false, false>;
+            auto kernel = bulk_pair_kernel<S, FORM, false, false, false>;
+            if constexpr (odd_pairs)
+                if (odd) kernel = bulk_pair_kernel<S, FORM, false, false, true>;
             // (the faces known at compile time where it pays: not beside the
             // exact stabilizer's arithmetic, nor beside single-element loads)
             if constexpr (FORM != FORM_MX) {
@@ -240,14 +247,15 @@ cudaError_t launch_bulk_form(const Lattice &L, const S *fa, S *fb, const uint8_t
     return cudaGetLastError();
 }
 
-// 16-bit boxes with a body and fewer nodes than this keep kbc_collide_v: their
-// step is bound by the body's chain and both forms take the same time (128x128x
-// 256 sphere), so the results of the 16-bit storage, whose rounding any other
-// operation order moves, stay bit for bit.  Larger ones and those without a
+// FP32 and 16-bit boxes with a body and fewer nodes than this keep
+// kbc_collide_v: their step is bound by the body's chain (and FP32's bulk launch
+// by memory), both forms take the same time (128x128x256 sphere), and what a
+// different operation order moves there shows in sums of both signs, such as
+// the mean thrust of an adjoint's objective.  Larger ones and those without a
 // body, where the bulk launch is the step, take kbc_collide_m (768x256x256
 // FP16 1219 -> 1062 us, 1024x512x64 with faces 874 -> 767).  A slab goes by the
 // whole box, whose bits its own layers have to give.
-constexpr long long MOMENT_FORM_NODES_16 = 1LL << 23;
+constexpr long long MOMENT_FORM_NODES = 1LL << 23;
 
 template <typename S>
 cudaError_t launch_bulk_t(const Lattice &L, const S *fa, S *fb, const uint8_t *flags, int *status, cudaStream_t s,
@@ -258,8 +266,8 @@ cudaError_t launch_bulk_t(const Lattice &L, const S *fa, S *fb, const uint8_t *f
     };
     constexpr bool dbl = std::is_same<S, double>::value;
     if (L.gamma_mode == LBM_GAMMA_EXACT) return form(std::integral_constant<int, dbl ? FORM_X : FORM_MX>{});
-    if constexpr (sizeof(S) == 2)
-        if (L.n_box < MOMENT_FORM_NODES_16 && (mode != BULK_ALL || flags)) return form(std::integral_constant<int, FORM_V>{});
+    if constexpr (!dbl)
+        if (L.n_box < MOMENT_FORM_NODES && (mode != BULK_ALL || flags)) return form(std::integral_constant<int, FORM_V>{});
     return form(std::integral_constant<int, FORM_M>{});
 }
 

@@ -239,74 +239,198 @@ __device__ __forceinline__ float det3f(const float a[3], const float b[3], const
     return a[0] * (b[1] * d[2] - b[2] * d[1]) - a[1] * (b[0] * d[2] - b[2] * d[0]) + a[2] * (b[0] * d[1] - b[1] * d[0]);
 }
 
-// Warp-cooperative form of the mesh link search for a boundary node: the
-// missing links (bits of mask) are taken one at a time by the whole warp;
-// each lane tests a strided share of the candidate triangles (same tests as
-// mesh_link for double, mesh_link_f for float), and a warp arg-min over
-// (s, triangle index) picks the first crossing.  Lane i receives q, u_w and
-// the hit of link i.  Every lane of the warp must call it.
+// A triangle relative to node p in single precision, from its vertices' split
+// positions: edges and the offset of p from the first vertex.
+struct TriF {
+    float e1[3], e2[3], r[3];
+    __device__ __forceinline__ TriF(const GeomParams &G, int k, const int p[3])
+    {
+        const int t0 = G.mesh_tris[3 * k], t1 = G.mesh_tris[3 * k + 1], t2 = G.mesh_tris[3 * k + 2];
+        for (int a = 0; a < 3; ++a) {
+            const float pa = (float)(G.mesh_ipos[3 * t0 + a] - p[a]) + G.mesh_frac[3 * t0 + a];
+            const float pb = (float)(G.mesh_ipos[3 * t1 + a] - p[a]) + G.mesh_frac[3 * t1 + a];
+            const float pc = (float)(G.mesh_ipos[3 * t2 + a] - p[a]) + G.mesh_frac[3 * t2 + a];
+            e1[a] = pb - pa;
+            e2[a] = pc - pa;
+            r[a] = -pa;
+        }
+    }
+    // crossing of the link from p along -c at p - sv c, with its barycentric
+    // coordinates
+    __device__ __forceinline__ bool hit(const int c[3], float &sv, float &uf, float &vf) const
+    {
+        constexpr float EPS = 1e-6f;
+        const float dc[3] = {(float)c[0], (float)c[1], (float)c[2]};
+        const float D = det3f(e1, e2, dc);
+        if (D == 0.0f) return false;
+        const float iD = 1.0f / D;
+        uf = det3f(r, e2, dc) * iD;
+        vf = det3f(e1, r, dc) * iD;
+        const float sf = det3f(e1, e2, r) * iD;
+        if (uf < -EPS || vf < -EPS || uf + vf > 1.0f + EPS || sf < -EPS || sf > 1.0f + EPS) return false;
+        sv = fminf(fmaxf(sf, 0.0f), 1.0f);
+        return true;
+    }
+};
+
+// a warp's scratch of the link search, in shared memory
+struct LinkScratch {
+    unsigned long long key[Q];  // per direction: (s, triangle index) of the first crossing
+    int start[8], cell[8];      // the cells to search: first position in their joint list, index
+    unsigned pair[64];          // triangle and link to be tested: 32 k + i
+};
+
+// First crossings of all missing links of a node (bits of mask) in single
+// precision.  The lists of the up to eight cells that the links' common box
+// overlaps are taken as one, 32 triangles at a time.  A triangle's box says per
+// axis which link components it can meet, their intersection which links; these
+// pairs (some ten a link of a hundred triangles looked at) are queued and tested
+// 32 at a time, and a link's first crossing, ties to the lower triangle index,
+// is the minimum of (s, index) in shared memory.  (One link after the other with
+// a warp arg-min each, or every triangle against every link, ran the test of 60
+// instructions with a few lanes at work: boundary kernel of the L = 64 swimmer 99
+// and 147 us.)
+__device__ __forceinline__ void mesh_first_crossings(const GeomParams &G, const DevBody *b, const int p[3],
+                                                     uint32_t mask, int lane, LinkScratch &S)
+{
+    // directions with c_a = +1 (their links end at p_a - 1) and -1, per axis
+    constexpr uint32_t ALL = (1u << Q) - 1u;
+    constexpr uint32_t PLUS[3] = {0x7FC0000u, 0x70381C0u, 0x4924924u};
+    constexpr uint32_t MINUS[3] = {0x1FFu, 0x1C0E07u, 0x1249249u};
+    int c0[3], nc[3];
+    for (int a = 0; a < 3; ++a) {
+        const int e0 = p[a] - ((mask & PLUS[a]) ? 1 : 0), e1 = p[a] + ((mask & MINUS[a]) ? 1 : 0);
+        // (three nodes span at most two cells of two)
+        c0[a] = max(0, (e0 - b->band_lo[a]) / MESH_CELL);
+        nc[a] = min(G.cells[a] - 1, (e1 - b->band_lo[a]) / MESH_CELL) - c0[a] + 1;
+    }
+    const int d[3] = {lane & 1, (lane >> 1) & 1, (lane >> 2) & 1};
+    int cell = 0, n = 0;
+    if (lane < 8 && d[0] < nc[0] && d[1] < nc[1] && d[2] < nc[2]) {
+        cell = (c0[0] + d[0]) + G.cells[0] * ((c0[1] + d[1]) + G.cells[1] * (c0[2] + d[2]));
+        n = min(G.cell_count[cell], MESH_CELL_CAP);
+    }
+    int end = n;
+    for (int o = 1; o < 8; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += t;
+    }
+    const int total = __shfl_sync(0xffffffffu, end, 7);
+    if (lane < 8) {
+        S.start[lane] = end - n;
+        S.cell[lane] = cell;
+    }
+    if (lane < Q) S.key[lane] = ~0ull;
+    __syncwarp();
+    const auto test = [&](unsigned pair) {
+        const int i = pair & 31, k = pair >> 5;
+        const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
+        float sv, u, v;
+        if (TriF(G, k, p).hit(c, sv, u, v))
+            atomicMin(S.key + i, (unsigned long long)__float_as_uint(sv + 0.0f) << 32 | (unsigned)k);
+    };
+    int queued = 0;
+    for (int j0 = 0; j0 < total; j0 += 32) {
+        const int j = j0 + lane;
+        int k = 0;
+        uint32_t links = 0;
+        if (j < total) {
+            int e = 0;
+#pragma unroll
+            for (int m = 1; m < 8; ++m) e = j >= S.start[m] ? m : e;
+            k = G.cell_tri[(size_t)S.cell[e] * MESH_CELL_CAP + (j - S.start[e])];
+            const float *bx = G.tri_box + 6 * (size_t)k;
+            links = mask;
+            for (int a = 0; a < 3; ++a) {
+                // link spans [p - 1, p] (c = +1), [p, p] and [p, p + 1] (c = -1)
+                const float l = bx[a], h = bx[3 + a], q = (float)p[a];
+                uint32_t can = 0;
+                if (h >= q - 1.0f && l <= q) can |= PLUS[a];
+                if (h >= q && l <= q) can |= ALL & ~(PLUS[a] | MINUS[a]);
+                if (h >= q && l <= q + 1.0f) can |= MINUS[a];
+                links &= can;
+            }
+        }
+        for (unsigned has = __ballot_sync(0xffffffffu, links != 0); has; has = __ballot_sync(0xffffffffu, links != 0)) {
+            if (links) {
+                S.pair[queued + __popc(has & ((1u << lane) - 1u))] = (unsigned)k << 5 | (unsigned)(__ffs(links) - 1);
+                links &= links - 1;
+            }
+            queued += __popc(has);
+            if (queued >= 32) {
+                __syncwarp();
+                queued -= 32;
+                const unsigned t = S.pair[queued + lane];
+                __syncwarp();
+                test(t);
+            }
+        }
+    }
+    __syncwarp();
+    if (lane < queued) test(S.pair[lane]);
+    __syncwarp();
+}
+
+// Warp-cooperative form of the mesh link search for a boundary node: lane i of
+// a missing link (bits of mask) receives its fraction q, wall velocity u_w and
+// hit.  Double: the links are taken one at a time by the whole warp, each lane
+// testing a strided share of the candidate triangles, and a warp arg-min over
+// (s, triangle index) picks the first crossing; single precision: see
+// mesh_first_crossings.  Every lane of the warp must call it; S: the warp's own.
 template <typename R>
 __device__ void mesh_links_warp(const GeomParams &G, const DevBody *b, int x, int y, int z, uint32_t mask, int lane,
-                                double &q, double uw[3], MeshHit &hitout)
+                                double &q, double uw[3], MeshHit &hitout, LinkScratch &S)
 {
-    constexpr bool single = sizeof(R) == 4;
     const int p[3] = {x, y, z};
-    const double *P = G.mesh_pos;
-    uint32_t m = mask;
-    while (m) {
-        const int i = __ffs(m) - 1;
-        m &= m - 1;
-        const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
-        int c0[3], c1[3];
-        float lo[3], hi[3];
-        for (int a = 0; a < 3; ++a) {
-            const int e0 = min(p[a], p[a] - c[a]), e1 = max(p[a], p[a] - c[a]);
-            lo[a] = (float)e0;
-            hi[a] = (float)e1;
-            c0[a] = max(0, (e0 - b->band_lo[a]) / MESH_CELL);
-            c1[a] = min(G.cells[a] - 1, (e1 - b->band_lo[a]) / MESH_CELL);
+    if constexpr (sizeof(R) == 4) {
+        mesh_first_crossings(G, b, p, mask, lane, S);
+        if ((mask >> lane) & 1u) {
+            const unsigned long long kk = S.key[lane];
+            if (kk != ~0ull) {
+                const int c[3] = {cx_of(lane), cy_of(lane), cz_of(lane)};
+                float sv = 0.f, u = 0.f, v = 0.f;
+                hitout.tri = (int)(unsigned)kk;
+                TriF(G, hitout.tri, p).hit(c, sv, u, v);
+                hitout.u = u;
+                hitout.v = v;
+                q = sv;
+            }
         }
-        // candidate values in the search precision (float coordinates relative
-        // to the node from the split vertex positions; double as in the oracle)
-        R best = R(2), bu = R(0), bv = R(0);
-        int bt = -1;
-        for (int kz = c0[2]; kz <= c1[2]; ++kz)
-            for (int ky = c0[1]; ky <= c1[1]; ++ky)
-                for (int kx = c0[0]; kx <= c1[0]; ++kx) {
-                    const int cell = kx + G.cells[0] * (ky + G.cells[1] * kz);
-                    const int n = min(G.cell_count[cell], MESH_CELL_CAP);
-                    const int *list = G.cell_tri + (size_t)cell * MESH_CELL_CAP;
-                    for (int j = lane; j < n; j += 32) {
-                        const int k = list[j];
-                        const float *bx = G.tri_box + 6 * (size_t)k;
-                        if (bx[3] < lo[0] || bx[0] > hi[0] || bx[4] < lo[1] || bx[1] > hi[1] || bx[5] < lo[2] ||
-                            bx[2] > hi[2])
-                            continue;
-                        const int t0 = G.mesh_tris[3 * k], t1 = G.mesh_tris[3 * k + 1], t2 = G.mesh_tris[3 * k + 2];
-                        R sv, u, v;
-                        if (single) {
-                            constexpr float EPS = 1e-6f;
-                            float A[3], e1[3], e2[3], r[3];
-                            for (int a = 0; a < 3; ++a) {
-                                const float pa = (float)(G.mesh_ipos[3 * t0 + a] - p[a]) + G.mesh_frac[3 * t0 + a];
-                                const float pb = (float)(G.mesh_ipos[3 * t1 + a] - p[a]) + G.mesh_frac[3 * t1 + a];
-                                const float pc = (float)(G.mesh_ipos[3 * t2 + a] - p[a]) + G.mesh_frac[3 * t2 + a];
-                                A[a] = pa;
-                                e1[a] = pb - pa;
-                                e2[a] = pc - pa;
-                                r[a] = -pa;
-                            }
-                            const float dc[3] = {(float)c[0], (float)c[1], (float)c[2]};
-                            const float D = det3f(e1, e2, dc);
-                            if (D == 0.0f) continue;
-                            const float iD = 1.0f / D;
-                            const float uf = det3f(r, e2, dc) * iD, vf = det3f(e1, r, dc) * iD;
-                            const float sf = det3f(e1, e2, r) * iD;
-                            if (uf < -EPS || vf < -EPS || uf + vf > 1.0f + EPS || sf < -EPS || sf > 1.0f + EPS) continue;
-                            sv = (R)fminf(fmaxf(sf, 0.0f), 1.0f);
-                            u = (R)uf;
-                            v = (R)vf;
-                        } else {
+        __syncwarp();
+    } else {
+        const double *P = G.mesh_pos;
+        uint32_t m = mask;
+        while (m) {
+            const int i = __ffs(m) - 1;
+            m &= m - 1;
+            const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
+            int c0[3], c1[3];
+            float lo[3], hi[3];
+            for (int a = 0; a < 3; ++a) {
+                const int e0 = min(p[a], p[a] - c[a]), e1 = max(p[a], p[a] - c[a]);
+                lo[a] = (float)e0;
+                hi[a] = (float)e1;
+                c0[a] = max(0, (e0 - b->band_lo[a]) / MESH_CELL);
+                c1[a] = min(G.cells[a] - 1, (e1 - b->band_lo[a]) / MESH_CELL);
+            }
+            // candidate values in the search precision (float coordinates relative
+            // to the node from the split vertex positions; double as in the oracle)
+            R best = R(2), bu = R(0), bv = R(0);
+            int bt = -1;
+            for (int kz = c0[2]; kz <= c1[2]; ++kz)
+                for (int ky = c0[1]; ky <= c1[1]; ++ky)
+                    for (int kx = c0[0]; kx <= c1[0]; ++kx) {
+                        const int cell = kx + G.cells[0] * (ky + G.cells[1] * kz);
+                        const int n = min(G.cell_count[cell], MESH_CELL_CAP);
+                        const int *list = G.cell_tri + (size_t)cell * MESH_CELL_CAP;
+                        for (int j = lane; j < n; j += 32) {
+                            const int k = list[j];
+                            const float *bx = G.tri_box + 6 * (size_t)k;
+                            if (bx[3] < lo[0] || bx[0] > hi[0] || bx[4] < lo[1] || bx[1] > hi[1] || bx[5] < lo[2] ||
+                                bx[2] > hi[2])
+                                continue;
+                            const int t0 = G.mesh_tris[3 * k], t1 = G.mesh_tris[3 * k + 1], t2 = G.mesh_tris[3 * k + 2];
+                            R sv, u, v;
                             double e1[3], e2[3], r[3];
                             for (int a = 0; a < 3; ++a) {
                                 e1[a] = P[3 * t1 + a] - P[3 * t0 + a];
@@ -323,33 +447,33 @@ __device__ void mesh_links_warp(const GeomParams &G, const DevBody *b, int x, in
                             sv = (R)sd;
                             u = (R)ud;
                             v = (R)vd;
-                        }
-                        if (sv < best || (sv == best && k < bt)) {
-                            best = sv;
-                            bt = k;
-                            bu = u;
-                            bv = v;
+                            if (sv < best || (sv == best && k < bt)) {
+                                best = sv;
+                                bt = k;
+                                bu = u;
+                                bv = v;
+                            }
                         }
                     }
+            // arg-min over the warp, ties to the lower triangle index
+            for (int o = 16; o > 0; o >>= 1) {
+                const R ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int ot = __shfl_xor_sync(0xffffffffu, bt, o);
+                const R ou = __shfl_xor_sync(0xffffffffu, bu, o);
+                const R ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                if (ot >= 0 && (bt < 0 || ob < best || (ob == best && ot < bt))) {
+                    best = ob;
+                    bt = ot;
+                    bu = ou;
+                    bv = ov;
                 }
-        // arg-min over the warp, ties to the lower triangle index
-        for (int o = 16; o > 0; o >>= 1) {
-            const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int ot = __shfl_xor_sync(0xffffffffu, bt, o);
-            const R ou = __shfl_xor_sync(0xffffffffu, bu, o);
-            const R ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            if (ot >= 0 && (bt < 0 || ob < best || (ob == best && ot < bt))) {
-                best = ob;
-                bt = ot;
-                bu = ou;
-                bv = ov;
             }
-        }
-        if (lane == i) {
-            hitout.tri = bt;
-            hitout.u = bu;
-            hitout.v = bv;
-            q = best;
+            if (lane == i) {
+                hitout.tri = bt;
+                hitout.u = bu;
+                hitout.v = bv;
+                q = best;
+            }
         }
     }
     // the wall velocities of all links at once (FP64: one pass of the pipe for

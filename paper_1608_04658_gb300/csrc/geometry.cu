@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, c
 // vertex positions x = X0 + s, y = (X1 + y(s,t)) + dy, z = X2 + dz (head
 // frame) or X + R(psi) (b - c(t)) (centre-of-mass frame, with the lattice box
 // of the pose) and velocities; clears the column and cell lists of the step.
-__global__ void __launch_bounds__(MESH_THREADS) mesh_pose_kernel(const Lattice L, const GeomParams G,
+__global__ void __launch_bounds__(POSE_THREADS) mesh_pose_kernel(const Lattice L, const GeomParams G,
                                                                  const DevBody *__restrict__ prev,
                                                                  DevBody *__restrict__ next, int advance,
                                                                  int ncols, int ncells)
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(MESH_THREADS) mesh_pose_kernel(const Lattice L
 
 // Per triangle: its box, the band columns whose line crosses it (with the
 // crossing abscissa) and the band cells its box overlaps.
-__global__ void __launch_bounds__(MESH_THREADS) mesh_bin_kernel(const Lattice L, const GeomParams G,
+__global__ void __launch_bounds__(POSE_THREADS) mesh_bin_kernel(const Lattice L, const GeomParams G,
                                                                 const DevBody *__restrict__ prev,
                                                                 const DevBody *__restrict__ next, int advance)
 {
@@ -791,12 +791,12 @@ cudaError_t launch_mesh_prepare(const Lattice &L, const GeomParams &G, Scratch &
 {
     const int ncols = G.cap[1] * G.cap[2];
     const int ncells = G.cells[0] * G.cells[1] * G.cells[2];
-    const int nb_v = (G.n_vertices + MESH_THREADS - 1) / MESH_THREADS;
-    const int nb_t = (G.n_triangles + MESH_THREADS - 1) / MESH_THREADS;
+    const int nb_v = (G.n_vertices + POSE_THREADS - 1) / POSE_THREADS;
+    const int nb_t = (G.n_triangles + POSE_THREADS - 1) / POSE_THREADS;
     DevBody *next = S.body + (advance ? prev ^ 1 : prev);
-    mesh_pose_kernel<<<nb_v > 0 ? nb_v : 1, MESH_THREADS, 0, s>>>(L, G, S.body + prev, next, advance ? 1 : 0, ncols,
+    mesh_pose_kernel<<<nb_v > 0 ? nb_v : 1, POSE_THREADS, 0, s>>>(L, G, S.body + prev, next, advance ? 1 : 0, ncols,
                                                                     ncells);
-    mesh_bin_kernel<<<nb_t > 0 ? nb_t : 1, MESH_THREADS, 0, s>>>(L, G, S.body + prev, next, advance ? 1 : 0);
+    mesh_bin_kernel<<<nb_t > 0 ? nb_t : 1, POSE_THREADS, 0, s>>>(L, G, S.body + prev, next, advance ? 1 : 0);
     *nlaunch += 2;
     return cudaGetLastError();
 }
