@@ -248,8 +248,10 @@ __device__ R kbc_vjp_lanes(R g, R lam, int i, R beta, R inv_beta, R rho0, int ga
     const int cx = act ? cx_of(i) : 0, cy = act ? cy_of(i) : 0, cz = act ? cz_of(i) : 0;
     const int nz = act ? nonzero_of(i) : 0;
     const R gv = act ? g : R(0), lv = act ? lam : R(0);
-    const R drho = wsum(gv);
-    const R jx = wsum(R(cx) * gv), jy = wsum(R(cy) * gv), jz = wsum(R(cz) * gv);
+    const int lane = threadIdx.x & 31;
+    R m4[4] = {gv, R(cx) * gv, R(cy) * gv, R(cz) * gv};
+    wsum4(m4, lane);
+    const R drho = m4[0], jx = m4[1], jy = m4[2], jz = m4[3];
     const R rho = rho0 + drho, irho = R(1) / rho;
     const R u[3] = {jx * irho, jy * irho, jz * irho};
     R e[3][3], phi[3][3], rr[3][3], dl[3][3];
@@ -257,14 +259,17 @@ __device__ R kbc_vjp_lanes(R g, R lam, int i, R beta, R inv_beta, R rho0, int ga
     const R exy = pick(e[0], cx) + pick(e[1], cy) + pick(e[0], cx) * pick(e[1], cy);
     const R E = exy + pick(e[2], cz) + exy * pick(e[2], cz);
     const R d = act ? gv - weight<R>(i) * (drho + rho * E) : R(0);
-    const R pxx = wsum(R(cx * cx) * d), pyy = wsum(R(cy * cy) * d), pzz = wsum(R(cz * cz) * d);
-    const R pxy = wsum(R(cx * cy) * d), pxz = wsum(R(cx * cz) * d), pyz = wsum(R(cy * cz) * d);
+    R p6[6] = {R(cx * cx) * d, R(cy * cy) * d, R(cz * cz) * d, R(cx * cy) * d, R(cx * cz) * d, R(cy * cz) * d};
+    wsum6(p6, lane);
+    const R pxx = p6[0], pyy = p6[1], pzz = p6[2], pxy = p6[3], pxz = p6[4], pyz = p6[5];
     const R nxz = pxx - pzz, nyz = pyy - pzz;
     const R ds = act ? shear_part_raw<R>(i, nxz, nyz, pxy, pxz, pyz) : R(0);
     const R dh = d - ds;
     const R ifeq = act ? irho * inv_weight<R>(i) * pick(rr[0], cx) * pick(rr[1], cy) * pick(rr[2], cz) : R(0);
     const R feq = act ? rho * weight<R>(i) * pick(phi[0], cx) * pick(phi[1], cy) * pick(phi[2], cz) : R(0);
-    const R sh = wsum(ds * dh * ifeq), hh = wsum(dh * dh * ifeq), lh = wsum(lv * dh);
+    R s4[4] = {ds * dh * ifeq, dh * dh * ifeq, lv * dh, R(0)};
+    wsum4(s4, lane);
+    const R sh = s4[0], hh = s4[1], lh = s4[2];
     const bool analytic = gamma_mode == LBM_GAMMA_ANALYTIC && hh > gamma_floor<R>();
     const R gam = analytic ? inv_beta - (R(2) - inv_beta) * sh / hh : R(2);
     const R gb = -beta * lh;
@@ -275,19 +280,20 @@ __device__ R kbc_vjp_lanes(R g, R lam, int i, R beta, R inv_beta, R rho0, int ga
     const R dsb = -R(2) * beta * lv + ab * dh * ifeq;
     const R dhb = -beta * gam * lv + ab * ds * ifeq + R(2) * bb * dh * ifeq;
     const R t = (nz == 1 || nz == 2) ? dsb - dhb : R(0);
-    const R Sx = wsum((nz == 1 && cx) ? t : R(0));
-    const R Sy = wsum((nz == 1 && cy) ? t : R(0));
-    const R Sz = wsum((nz == 1 && cz) ? t : R(0));
-    const R Qxy = wsum((nz == 2 && cz == 0) ? R(cx * cy) * t : R(0));
-    const R Qxz = wsum((nz == 2 && cy == 0) ? R(cx * cz) * t : R(0));
-    const R Qyz = wsum((nz == 2 && cx == 0) ? R(cy * cz) * t : R(0));
+    R t6[6] = {(nz == 1 && cx) ? t : R(0), (nz == 1 && cy) ? t : R(0), (nz == 1 && cz) ? t : R(0),
+               (nz == 2 && cz == 0) ? R(cx * cy) * t : R(0), (nz == 2 && cy == 0) ? R(cx * cz) * t : R(0),
+               (nz == 2 && cx == 0) ? R(cy * cz) * t : R(0)};
+    wsum6(t6, lane);
+    const R Sx = t6[0], Sy = t6[1], Sz = t6[2], Qxy = t6[3], Qxz = t6[4], Qyz = t6[5];
     const R nxzb = (R(2) * Sx - Sy - Sz) * R(1.0 / 6.0);
     const R nyzb = (R(2) * Sy - Sx - Sz) * R(1.0 / 6.0);
     const R dfb = dhb + nxzb * R(cx * cx) + nyzb * R(cy * cy) - (nxzb + nyzb) * R(cz * cz) +
                   R(0.25) * (Qxy * R(cx * cy) + Qxz * R(cx * cz) + Qyz * R(cy * cz));
     const R tf = act ? -(ab * ds * dh + bb * dh * dh) * ifeq - dfb * feq : R(0);
-    R rhob = wsum(tf) * irho;
-    const R ub[3] = {wsum(tf * pick(dl[0], cx)), wsum(tf * pick(dl[1], cy)), wsum(tf * pick(dl[2], cz))};
+    R u4[4] = {tf, tf * pick(dl[0], cx), tf * pick(dl[1], cy), tf * pick(dl[2], cz)};
+    wsum4(u4, lane);
+    R rhob = u4[0] * irho;
+    const R ub[3] = {u4[1], u4[2], u4[3]};
     rhob -= (ub[0] * u[0] + ub[1] * u[1] + ub[2] * u[2]) * irho;
     if (!act) return R(0);
     return lv + dfb + rhob + (R(cx) * ub[0] + R(cy) * ub[1] + R(cz) * ub[2]) * irho;
@@ -683,18 +689,15 @@ __device__ __forceinline__ void grad_pressure_adj(R gb, int i, bool act, R rho, 
     const R cx = act ? R(cx_of(i)) : R(0), cy = act ? R(cy_of(i)) : R(0), cz = act ? R(cz_of(i)) : R(0);
     const R w = act ? weight<R>(i) * gb : R(0);
     const R cu = cx * u[0] + cy * u[1] + cz * u[2];
-    rhob += wsum(w * (R(1) + R(3) * cu));
-    ub[0] += wsum(w * R(3) * rho * cx);
-    ub[1] += wsum(w * R(3) * rho * cy);
-    ub[2] += wsum(w * R(3) * rho * cz);
+    const int lane = threadIdx.x & 31;
+    R m4[4] = {w * (R(1) + R(3) * cu), w * R(3) * rho * cx, w * R(3) * rho * cy, w * R(3) * rho * cz};
+    wsum4(m4, lane);
+    rhob += m4[0];
+    for (int a = 0; a < 3; ++a) ub[a] += m4[1 + a];
     const R third = R(1.0 / 3.0);
-    R Qb[6];
-    Qb[0] = wsum(w * R(4.5) * (cx * cx - third));
-    Qb[1] = wsum(w * R(4.5) * (cy * cy - third));
-    Qb[2] = wsum(w * R(4.5) * (cz * cz - third));
-    Qb[3] = wsum(w * R(9) * cx * cy);
-    Qb[4] = wsum(w * R(9) * cx * cz);
-    Qb[5] = wsum(w * R(9) * cy * cz);
+    R Qb[6] = {w * R(4.5) * (cx * cx - third), w * R(4.5) * (cy * cy - third), w * R(4.5) * (cz * cz - third),
+               w * R(9) * cx * cy, w * R(9) * cx * cz, w * R(9) * cy * cz};
+    wsum6(Qb, lane);
     // Qt_ab = rho u_a u_b - (rho / (6 beta)) (du_ab + du_ba)
     const R k6 = R(1) / (R(6) * beta);
     const int A[6] = {0, 1, 2, 0, 0, 1}, B[6] = {0, 1, 2, 1, 2, 2};
@@ -731,16 +734,17 @@ constexpr int BODY_SLOTS = 12;
 // (same operations as the boundary kernel), then its transpose.
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
-    const Lattice L, const GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ blist,
+    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ blist,
     const int *__restrict__ bpos, const S *__restrict__ st, const NextAdj<typename Codec<S>::R> A,
     const uint8_t *__restrict__ flags1, typename Codec<S>::R *__restrict__ lam_out, double *__restrict__ ext,
     double *__restrict__ tslots, const BodyAdjoint *__restrict__ badj, double *__restrict__ bslot,
     const ComTangents *__restrict__ ct)
 {
     using R = typename Codec<S>::R;
-    __shared__ R s_f[BWARPS][Q][28];
+    __shared__ __align__(16) R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
     __shared__ LinkScratch s_link[BWARPS];
+    __shared__ WallMotion<R> s_wall;
     __shared__ int s_ok[BWARPS][Q];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     R (*sf)[28] = s_f[w];
@@ -752,52 +756,37 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
     const double fw[3] = {badj->fw[0], badj->fw[1], badj->fw[2]};
     const double mw = badj->mw;
 
+    s_wall.load(G, b);
+    const int i = lane;
+    const bool act = i < Q;
+    const int cx = act ? cx_of(i) : 0, cy = act ? cy_of(i) : 0, cz = act ? cz_of(i) : 0;
+    const int off = direction_offset(L, act ? i : 13);
+
     for (int slot = blockIdx.x * BWARPS + w; slot < count; slot += gridDim.x * BWARPS) {
         const int n = blist[slot];
         int x, y, z;
         node_xyz(L, n, x, y, z);
-        const int i = lane;
-        const bool act = i < Q;
-        const int cx = act ? cx_of(i) : 0, cy = act ? cy_of(i) : 0, cz = act ? cz_of(i) : 0;
-        bool solid_src = false;
-        if (act && i != 13) {
-            const int src = pull_source(L, x, y, z, cx, cy, cz);
-            solid_src = src >= 0 && (flags1[src] & FL_SOLID);
-        }
-        const uint32_t mask = __ballot_sync(FULL, solid_src);
-        int nk = -1;
-        if (act) nk = neighbour(L, x, y, z, cx, cy, cz);
-        if (act) sok[lane] = nk >= 0 && !(flags1[nk] & FL_SOLID);
+        int nk, src;
+        const uint32_t mask = node_links(L, flags1, n, x, y, z, lane, off, sok, nk, src);
+        const bool miss = act && ((mask >> i) & 1u);
+        // known pulls (face rules as in the bulk kernel)
+        R Fi = R(0);
+        if (act && !miss && src >= 0) Fi = Codec<S>::load(st + (size_t)i * N + src);
         __syncwarp();
         const uint32_t need = (1u << 13) | (1u << 22) | (1u << 4) | (1u << 16) | (1u << 10) |
                               (1u << 14) | (1u << 12) | mask;
         stage<S, R>(L, st, lane, nk, need, sf, su, sok);
-        const bool miss = act && ((mask >> i) & 1u);
-        // known pulls (face rules as in the bulk kernel)
-        R Fi = R(0);
-        if (act && !miss) {
-            int p[3] = {x - cx, y - cy, z - cz};
-            const int nn[3] = {L.nx, L.ny, L.nz};
-            int kind = 0;
-            for (int a = 0; a < 3; ++a) {
-                int face = -1;
-                if (p[a] < 0) face = L.face[2 * a];
-                else if (p[a] >= nn[a]) face = L.face[2 * a + 1];
-                if (face < 0) continue;
-                if (face == LBM_FACE_PERIODIC) p[a] = (p[a] + nn[a]) % nn[a];
-                else if (face == LBM_FACE_OUTFLOW) p[a] = p[a] < 0 ? 0 : nn[a] - 1;
-                else if (face == LBM_FACE_WALL) kind = 2;
-                else kind = kind > 1 ? kind : 1;
-            }
-            if (kind == 2) Fi = sf[13][26 - i];
-            else if (kind == 1) Fi = (R)L.g_face[i];
-            else Fi = Codec<S>::load(st + (size_t)i * N + (p[0] + L.nx * (p[1] + L.ny * p[2])));
-        }
+        if (act && !miss && src < 0) Fi = src == -2 ? sf[13][26 - i] : (R)L.g_face[i];
         const R fbb = act ? sf[13][26 - (act ? i : 0)] : R(0);
         double q = 0, uw[3] = {0, 0, 0};
         MeshHit hit{-1, 0.0, 0.0};
         if (G.kind == LBM_BODY_MESH) mesh_links_warp<R>(G, b, x, y, z, mask, lane, q, uw, hit, s_link[w]);
-        else if (miss) link_data<R>(L, G, b, x, y, z, cx, cy, cz, q, uw);
+        else if (miss) {
+            R uh[3] = {s_wall.U[0], s_wall.U[1], s_wall.U[2]};
+            float ul[3] = {s_wall.lo[0], s_wall.lo[1], s_wall.lo[2]};
+            link_data<R>(L, G, b, s_wall.air, x, y, z, i, q, uh, ul);
+            for (int a = 0; a < 3; ++a) uw[a] = (double)uh[a] + (double)ul[a];
+        }
         const R gstat = miss ? fbb : Fi;
         const R dyn = miss ? R(6) * weight<R>(i) * rho0 * (R(cx) * (R)uw[0] + R(cy) * (R)uw[1] + R(cz) * (R)uw[2])
                            : R(0);
@@ -811,9 +800,10 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
             }
         }
         const R nmiss = R(__popc(mask));
-        const R rho_t = rho0 + wsum(act ? gstat : R(0)) + wsum(dyn);
-        R u_t[3];
-        for (int a = 0; a < 3; ++a) u_t[a] = wsum(ut[a]) / nmiss;
+        R ts[6] = {act ? gstat : R(0), dyn, ut[0], ut[1], ut[2], R(0)};
+        wsum6(ts, lane);
+        const R rho_t = rho0 + ts[0] + ts[1];
+        const R u_t[3] = {ts[2] / nmiss, ts[3] / nmiss, ts[4] / nmiss};
         R du[3][3];
         const R uc[3] = {su[13][1], su[13][2], su[13][3]};
         fd_gradient<R>(su, sok, uc, du);
@@ -944,18 +934,15 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
             for (int k = 0; k < 2; ++k) tb[k] = qb * dq[k] + uwb[1] * dU1[k];
         }
         // per-node sums over the links in R; the slots sum the nodes in double
-        for (int k = 0; k < 3; ++k) {
-            R v = (R)tb[k];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-            if (lane == 0) tslots[(size_t)bpos[slot] * 6 + k] += (double)v;
-        }
+        R t4[4] = {(R)tb[0], (R)tb[1], (R)tb[2], R(0)};
+        wsum4(t4, lane);
+        if (lane < 3) tslots[(size_t)bpos[slot] * 6 + lane] += (double)(lane == 0 ? t4[0] : lane == 1 ? t4[1] : t4[2]);
         // the free body's state through q and u_w of each missing link
         if (bslot) {
-            for (int d = 0; d < 6; ++d) {
-                double v = gb[d];
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-                if (lane == 0) bslot[(size_t)bpos[slot] * BODY_SLOTS + d] = v;
-            }
+            const double v = wsum_scatter6(gb, lane);
+#pragma unroll
+            for (int d = 0; d < 6; ++d)
+                if (lane == wsum_owner6(d)) bslot[(size_t)bpos[slot] * BODY_SLOTS + d] = v;
         }
         __syncwarp();
     }
@@ -966,13 +953,13 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
 // gradient), fed by lambda(St^t) at the node.
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32) adjoint_refill_kernel(
-    const Lattice L, const GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ ulist,
+    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ ulist,
     const int *__restrict__ upos, const S *__restrict__ st, const typename Codec<S>::R *__restrict__ lam_t,
     const uint8_t *__restrict__ flags1, double *__restrict__ ext, double *__restrict__ tslots,
     double *__restrict__ bslot, const ComTangents *__restrict__ ct)
 {
     using R = typename Codec<S>::R;
-    __shared__ R s_f[BWARPS][Q][28];
+    __shared__ __align__(16) R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
     __shared__ int s_ok[BWARPS][Q];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -991,7 +978,7 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_refill_kernel(
         if (act) sok[lane] = nk >= 0 && !(flags1[nk] & FL_SOLID_PREV);
         __syncwarp();
         const uint32_t need = __ballot_sync(FULL, act && sok[lane]);
-        stage<S, R>(L, st, lane, nk, need, sf, su, sok);
+        stage<S, R, true>(L, st, lane, nk, need, sf, su, sok);
         const R cnt = R(__popc(need));
         const R rsum = wsum((act && sok[lane]) ? su[lane][0] : R(0));
         const R rho = cnt > R(0) ? rsum / cnt : rho0;

@@ -11,6 +11,13 @@
 // shuffle trees whose lane-0 result is broadcast, so every lane sees the same
 // density, velocity and stabilizer.
 //
+// Bound by instructions and their latency (3000 a node, a twentieth of the DRAM
+// rate): the sources of an inner node from one mark a lane, 15 staged nodes for
+// 27, a link search of five or six evaluations for 24 and no conversion of the
+// wall's velocity per node took the 1024x512x64 airfoil's from 142 to 117 us
+// (16,000 nodes); a body of a few hundred nodes waits for its instructions (a
+// warp passes through once: 21 us for 300 nodes, before and after).
+//
 // Readings of points the paper leaves open (the oracle takes the same ones):
 //   missing set D = {i : x_b - c_i solid at t+1}; wall point x_w = x_b - q_i c_i;
 //   u_f,i from the previous-step state at x_b + c_i, or the wall velocity alone
@@ -43,10 +50,11 @@ namespace lbm {
 // time (airfoil 225 us with it).  The force kernel does it for 32 nodes a warp.
 template <typename R>
 __device__ __forceinline__ void node_force(double *__restrict__ slot, int lane, bool link, int cx, int cy, int cz,
-                                           int i, R fbb, R gi, double q, const double uw[3]);
+                                           int i, R fbb, R gi, R q, const R uw[3], const float ul[3]);
 template <>
 __device__ __forceinline__ void node_force<double>(double *__restrict__ slot, int lane, bool link, int cx, int cy,
-                                                   int cz, int i, double fbb, double gi, double q, const double uw[3])
+                                                   int cz, int i, double fbb, double gi, double q, const double uw[3],
+                                                   const float ul[3])
 {
     // force without W rho0, and -sum q (f_in - f_out) (c x u_w)
     double v[6] = {0, 0, 0, 0, 0, 0};
@@ -70,127 +78,129 @@ __device__ __forceinline__ void node_force<double>(double *__restrict__ slot, in
 }
 template <>
 __device__ __forceinline__ void node_force<float>(double *__restrict__ slot, int lane, bool link, int cx, int cy,
-                                                  int cz, int i, float fbb, float gi, double q, const double uw[3])
+                                                  int cz, int i, float fbb, float gi, float q, const float uw[3],
+                                                  const float ul[3])
 {
     Pair32 F[3] = {};
     float H[3] = {0.f, 0.f, 0.f};
     if (link) {
         const Pair32 sum = two_sum(fbb, gi), dif = two_sum(gi, -fbb);
         const int c[3] = {cx, cy, cz};
-        float u[3];
         for (int a = 0; a < 3; ++a) {
-            u[a] = (float)uw[a];
-            const Pair32 p = Pair32{u[a], (float)(uw[a] - (double)u[a])} * dif;
+            const Pair32 p = Pair32{uw[a], ul[a]} * dif;
             F[a] = c[a] == 0 ? p : (c[a] > 0 ? p - sum : p + sum);
         }
-        const float h = -(float)q * dif.hi;
+        const float h = -q * dif.hi;
         for (int a = 0; a < 3; ++a) {
             const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
-            H[a] = h * (c[b1] * u[b2] - c[b2] * u[b1]);
+            H[a] = h * (c[b1] * uw[b2] - c[b2] * uw[b1]);
         }
     }
-    for (int o = 16; o > 0; o >>= 1)
+    // sums as in wsum_scatter6: component 2 to the upper half of the warp, 1 to
+    // the upper quarter of the lower half
+    const auto exchange = [&](Pair32 a, Pair32 b, int o) {
+        const bool up = lane & o;
+        const Pair32 keep = up ? b : a, send = up ? a : b;
+        return keep + Pair32{__shfl_xor_sync(FULL, send.hi, o), __shfl_xor_sync(FULL, send.lo, o)};
+    };
+    const Pair32 none = {0.f, 0.f}, F02 = exchange(F[0], F[2], 16), F1 = exchange(F[1], none, 16);
+    const float H02 = wexchange(H[0], H[2], lane, 16), H1 = wexchange(H[1], 0.f, lane, 16);
+    Pair32 Fs = exchange(F02, F1, 8);
+    float Hs = wexchange(H02, H1, lane, 8);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const Pair32 t = {__shfl_xor_sync(FULL, F[a].hi, o), __shfl_xor_sync(FULL, F[a].lo, o)};
-            F[a] = F[a] + t;
-            H[a] += __shfl_xor_sync(FULL, H[a], o);
-        }
+    for (int o = 4; o > 0; o >>= 1) {
+        Fs = Fs + Pair32{__shfl_xor_sync(FULL, Fs.hi, o), __shfl_xor_sync(FULL, Fs.lo, o)};
+        Hs += __shfl_xor_sync(FULL, Hs, o);
+    }
     const int w = link ? weight216(i) : 0;
     const int k0 = __reduce_add_sync(FULL, w * cx), k1 = __reduce_add_sync(FULL, w * cy),
               k2 = __reduce_add_sync(FULL, w * cz);
-    if (lane < 3) {
-        ForceSlot<float> *p = reinterpret_cast<ForceSlot<float> *>(slot);
-        p->hi[lane] = lane == 0 ? F[0].hi : (lane == 1 ? F[1].hi : F[2].hi);
-        p->lo[lane] = lane == 0 ? F[0].lo : (lane == 1 ? F[1].lo : F[2].lo);
-        p->h[lane] = lane == 0 ? H[0] : (lane == 1 ? H[1] : H[2]);
-        if (lane == 0) p->k = pack_k(k0, k1, k2);
+    ForceSlot<float> *p = reinterpret_cast<ForceSlot<float> *>(slot);
+    if ((lane & 7) == 0 && lane < 24) {
+        const int a = lane >> 3;  // lane 0, 8, 16: components 0, 1, 2
+        p->hi[a] = Fs.hi;
+        p->lo[a] = Fs.lo;
+        p->h[a] = Hs;
     }
+    if (lane == 0) p->k = pack_k(k0, k1, k2);
 }
 
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_kernel(
-    const Lattice L, const GeomParams G, DevBody *__restrict__ b, const int *__restrict__ blist,
+    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, DevBody *__restrict__ b, const int *__restrict__ blist,
     const int *__restrict__ bpos, double *__restrict__ bforce, const S *__restrict__ fa,
     S *__restrict__ fb, const uint8_t *__restrict__ flags)
 {
     using R = typename Codec<S>::R;
-    __shared__ R s_f[BWARPS][Q][28];
+    __shared__ __align__(16) R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
     __shared__ LinkScratch s_link[BWARPS];
+    __shared__ WallMotion<R> s_wall;
     __shared__ int s_ok[BWARPS][Q];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     R (*sf)[28] = s_f[w];
     R (*su)[4] = s_u[w];
     int *sok = s_ok[w];
+    // (the first node of the warp is read beside the count, not after it; the list
+    // has room for every warp that passes this check)
+    const int first = blockIdx.x * BWARPS + w;
+    int n = first < G.cap_boundary ? blist[first] : 0;
     const int count = min(b->n_boundary, G.cap_boundary);
     const size_t N = (size_t)L.N;
     const R rho0 = (R)L.rho0;
 
-    for (int slot = blockIdx.x * BWARPS + w; slot < count; slot += gridDim.x * BWARPS) {
-        const int n = blist[slot];
+    s_wall.load(G, b);
+    const int i = lane;
+    const bool act = i < Q;
+    const int cx = act ? cx_of(i) : 0, cy = act ? cy_of(i) : 0, cz = act ? cz_of(i) : 0;
+    const int off = direction_offset(L, act ? i : 13);
+
+    for (int slot = first; slot < count; slot += gridDim.x * BWARPS) {
+        if (slot != first) n = blist[slot];
         int x, y, z;
         node_xyz(L, n, x, y, z);
-        const int i = lane;
-        const bool act = i < Q;
-        const int cx = act ? cx_of(i) : 0, cy = act ? cy_of(i) : 0, cz = act ? cz_of(i) : 0;
-        // missing set: directions whose pull source is solid at t+1
-        bool solid_src = false;
-        if (act && i != 13) {
-            const int src = pull_source(L, x, y, z, cx, cy, cz);
-            solid_src = src >= 0 && (flags[src] & FL_SOLID);
-        }
-        const uint32_t mask = __ballot_sync(FULL, solid_src);
-
+        // missing set: directions whose pull source is solid at t+1;
         // neighbourhood node k = lane: x_b + c_k
-        int nk = -1;
-        if (act) nk = neighbour(L, x, y, z, cx, cy, cz);
-        if (act) sok[lane] = nk >= 0 && !(flags[nk] & FL_SOLID);
+        int nk, src;
+        const uint32_t mask = node_links(L, flags, n, x, y, z, lane, off, sok, nk, src);
+        const bool miss = act && ((mask >> i) & 1u);
+        // known pulled populations (face rules as in the bulk kernel)
+        R Fi = R(0);
+        if (act && !miss && src >= 0) Fi = Codec<S>::load(fa + (size_t)i * N + src);
         __syncwarp();
         const uint32_t need = (1u << 13) | (1u << 22) | (1u << 4) | (1u << 16) | (1u << 10) |
                               (1u << 14) | (1u << 12) | mask;
         stage<S, R>(L, fa, lane, nk, need, sf, su, sok);
-
-        const bool miss = act && ((mask >> i) & 1u);
-        // known pulled populations (face rules as in the bulk kernel)
-        R Fi = R(0);
-        if (act && !miss) {
-            int p[3] = {x - cx, y - cy, z - cz};
-            const int nn[3] = {L.nx, L.ny, L.nz};
-            int kind = 0;
-            for (int a = 0; a < 3; ++a) {
-                int face = -1;
-                if (p[a] < 0) face = L.face[2 * a];
-                else if (p[a] >= nn[a]) face = L.face[2 * a + 1];
-                if (face < 0) continue;
-                if (face == LBM_FACE_PERIODIC) p[a] = (p[a] + nn[a]) % nn[a];
-                else if (face == LBM_FACE_OUTFLOW) p[a] = p[a] < 0 ? 0 : nn[a] - 1;
-                else if (face == LBM_FACE_WALL) kind = 2;
-                else kind = kind > 1 ? kind : 1;
-            }
-            if (kind == 2) Fi = sf[13][26 - i];
-            else if (kind == 1) Fi = (R)L.g_face[i];
-            else Fi = Codec<S>::load(fa + (size_t)i * N + (p[0] + L.nx * (p[1] + L.ny * p[2])));
-        }
+        if (act && !miss && src < 0) Fi = src == -2 ? sf[13][26 - i] : (R)L.g_face[i];
         // target density and velocity over the missing set
         const R fbb = act ? sf[13][26 - (act ? i : 0)] : R(0);  // shifted f'_{opp i}(x_b, t)
-        double q = 0, uw[3] = {0, 0, 0};
+        double q = 0;
+        R uw[3] = {0, 0, 0};
+        float ul[3] = {0, 0, 0};
         if (G.kind == LBM_BODY_MESH) {
             MeshHit hit{-1, 0.0, 0.0};
-            mesh_links_warp<R>(G, b, x, y, z, mask, lane, q, uw, hit, s_link[w]);
+            double ud[3] = {0, 0, 0};
+            mesh_links_warp<R>(G, b, x, y, z, mask, lane, q, ud, hit, s_link[w]);
+            for (int a = 0; a < 3; ++a) {
+                uw[a] = (R)ud[a];
+                ul[a] = (float)(ud[a] - (double)uw[a]);
+            }
         } else if (miss) {
-            link_data<R>(L, G, b, x, y, z, cx, cy, cz, q, uw);
+            for (int a = 0; a < 3; ++a) {
+                uw[a] = s_wall.U[a];
+                ul[a] = s_wall.lo[a];
+            }
+            link_data<R>(L, G, b, s_wall.air, x, y, z, i, q, uw, ul);
         }
+        const R qq = (R)q;
         const R gstat = miss ? fbb : Fi;
-        const R dyn = miss ? R(6) * weight<R>(i) * rho0 * (R(cx) * (R)uw[0] + R(cy) * (R)uw[1] + R(cz) * (R)uw[2])
-                           : R(0);
+        const R dyn = miss ? R(6) * weight<R>(i) * rho0 * (R(cx) * uw[0] + R(cy) * uw[1] + R(cz) * uw[2]) : R(0);
         R ut[3] = {0, 0, 0};
         if (miss) {
-            const R qq = (R)q;
             if (sok[i]) {
-                for (int a = 0; a < 3; ++a) ut[a] = (qq * su[i][1 + a] + (R)uw[a]) / (R(1) + qq);
+                for (int a = 0; a < 3; ++a) ut[a] = (qq * su[i][1 + a] + uw[a]) / (R(1) + qq);
             } else {
-                for (int a = 0; a < 3; ++a) ut[a] = (R)uw[a];
+                for (int a = 0; a < 3; ++a) ut[a] = uw[a];
             }
         }
         const R nmiss = R(__popc(mask));
@@ -212,7 +222,7 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
         // into its band slot, which the force kernel turns into force and torque
         // a slab's links count where it owns the fluid node
         const bool own = z >= G.own_lo && z < G.own_hi;
-        node_force<R>(bforce + (size_t)bpos[slot] * FORCE_SLOT, lane, own && miss, cx, cy, cz, i, fbb, gi, q, uw);
+        node_force<R>(bforce + (size_t)bpos[slot] * FORCE_SLOT, lane, own && miss, cx, cy, cz, i, fbb, gi, qq, uw, ul);
 
         bool ok;
         const R out = kbc_collide_lanes<R>(gi, i, (R)L.beta, (R)L.inv_beta, rho0, L.gamma_mode, ok);
@@ -224,11 +234,11 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
 
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) refill_kernel(
-    const Lattice L, const GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ ulist,
+    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ ulist,
     S *__restrict__ fa, const uint8_t *__restrict__ flags)
 {
     using R = typename Codec<S>::R;
-    __shared__ R s_f[BWARPS][Q][28];
+    __shared__ __align__(16) R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
     __shared__ int s_ok[BWARPS][Q];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -249,7 +259,7 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) refill_kerne
         if (act) sok[lane] = nk >= 0 && !(flags[nk] & FL_SOLID_PREV);
         __syncwarp();
         uint32_t need = __ballot_sync(FULL, act && sok[lane]);
-        stage<S, R>(L, fa, lane, nk, need, sf, su, sok);
+        stage<S, R, true>(L, fa, lane, nk, need, sf, su, sok);
         const R cnt = R(__popc(need));
         const R rsum = wsum((act && sok[lane]) ? su[lane][0] : R(0));
         const R rho = cnt > R(0) ? rsum / cnt : rho0;

@@ -491,9 +491,7 @@ __device__ void mesh_links_warp(const GeomParams &G, const DevBody *b, int x, in
     }
 }
 
-// airfoil link in the chord frame: node position and link direction in
-// double, the 24 halvings in float with reciprocal constants
-// (airfoil_margin_f: half thickness less the distance from the camber line)
+// half thickness less the distance from the camber line (chord units)
 __device__ __forceinline__ float airfoil_margin_f(const GeomParams &G, float xi, float eta)
 {
     const float p = G.camber_p_f;
@@ -504,26 +502,66 @@ __device__ __forceinline__ float airfoil_margin_f(const GeomParams &G, float xi,
     return t - fabsf(eta - yc);
 }
 
-__device__ __forceinline__ bool inside_airfoil_f(const GeomParams &G, float xi, float eta)
-{
-    if (xi < 0.0f || xi > 1.0f) return false;
-    return airfoil_margin_f(G, xi, eta) > 0.0f;
-}
-
-__device__ __forceinline__ double link_airfoil_f(const GeomParams &G, const DevBody *b, int x, int y, int cx, int cy)
-{
-    const double dx = (double)x - b->X[0], dy = (double)y - b->X[1];
-    const float xi0 = (float)((dx * G.ca - dy * G.sa) * G.inv_chord);
-    const float eta0 = (float)((dx * G.sa + dy * G.ca) * G.inv_chord);
-    const float dxi = (float)(-(cx * G.ca - cy * G.sa) * G.inv_chord);
-    const float deta = (float)(-(cx * G.sa + cy * G.ca) * G.inv_chord);
-    float lo = 0.0f, hi = 1.0f;
-    for (int it = 0; it < 24; ++it) {
-        const float mid = 0.5f * (lo + hi);
-        if (inside_airfoil_f(G, xi0 + mid * dxi, eta0 + mid * deta)) hi = mid;
-        else lo = mid;
+// an airfoil link's direction and a node's position in the chord frame (chord
+// units): dxi, deta per direction; xi0 = x X[0] + y X[1] + X[2], eta0 likewise
+struct AirfoilFrame {
+    double X[3], Y[3];
+    float dxi[Q], deta[Q];
+    __device__ __forceinline__ void origin(const GeomParams &G, const DevBody *b)
+    {
+        X[0] = Y[1] = G.ca * G.inv_chord;
+        X[1] = -G.sa * G.inv_chord;
+        Y[0] = G.sa * G.inv_chord;
+        X[2] = -(b->X[0] * X[0] + b->X[1] * X[1]);
+        Y[2] = -(b->X[0] * Y[0] + b->X[1] * Y[1]);
     }
-    return (double)lo + 0x1p-25;  // the middle of [lo, lo + 2^-24]
+    __device__ __forceinline__ void direction(const GeomParams &G, int i)
+    {
+        const int cx = cx_of(i), cy = cy_of(i);
+        dxi[i] = (float)(-(cx * G.ca - cy * G.sa) * G.inv_chord);
+        deta[i] = (float)(-(cx * G.sa + cy * G.ca) * G.inv_chord);
+    }
+};
+
+// Crossing s in [0, 1] of a link from outside (s = 0) with the outline: false
+// position on the margin with the stale end's value halved (the Illinois
+// method; Dowell and Jarratt, BIT 11, 1971), five or six evaluations where
+// halving the interval to the same 2^-24 takes 24, each a square root and a
+// quartic deep: a quarter of the airfoil's boundary kernel.  A halving where the
+// lower end lies off the chord (the margin has no value there) and every fourth
+// time, which bounds the search.
+__device__ __forceinline__ double link_airfoil_f(const GeomParams &G, const AirfoilFrame &A, int x, int y, int i)
+{
+    const float xi0 = (float)fma((double)x, A.X[0], fma((double)y, A.X[1], A.X[2]));
+    const float eta0 = (float)fma((double)x, A.Y[0], fma((double)y, A.Y[1], A.Y[2]));
+    const float dxi = A.dxi[i], deta = A.deta[i];
+    const auto margin = [&](float s) {
+        const float xi = xi0 + s * dxi;
+        return xi < 0.0f || xi > 1.0f ? -INFINITY : airfoil_margin_f(G, xi, eta0 + s * deta);
+    };
+    float lo = 0.0f, hi = 1.0f, flo = margin(0.0f), fhi = margin(1.0f), s = 0.5f;
+    if (flo > 0.0f) return 0x1p-25;        // (the marks are the double decisions)
+    if (!(fhi > 0.0f)) return 1.0 - 0x1p-25;
+    int side = 0;
+    for (int it = 0; it < 64 && hi - lo > 0x1p-24f; ++it) {
+        const float last = s;
+        s = (it & 3) == 3 || flo == -INFINITY ? 0.5f * (lo + hi) : fmaf(hi - lo, __fdividef(flo, flo - fhi), lo);
+        s = fminf(fmaxf(s, lo), hi);
+        const float f = margin(s);
+        if (f > 0.0f) {
+            hi = s;
+            fhi = f;
+            if (side > 0) flo *= 0.5f;
+            side = 1;
+        } else {
+            lo = s;
+            flo = f;
+            if (side < 0) fhi *= 0.5f;
+            side = -1;
+        }
+        if ((it & 3) != 3 && it > 0 && fabsf(s - last) <= 0x1p-24f) break;
+    }
+    return (double)s;
 }
 
 // Pull source x - c under the box rules; node index, or -1 when a wall or
@@ -560,23 +598,46 @@ __device__ __forceinline__ int neighbour(const Lattice &L, int x, int y, int z, 
     return p[0] + L.nx * (p[1] + L.ny * p[2]);
 }
 
-// Link of boundary node (x, y, z) towards the solid node x - c: fraction q of
-// the link at which the wall is crossed (wall point x_w = x - q c, q in (0,1])
-// and the wall velocity there.  R is the collision arithmetic: double keeps
-// the plain double evaluation; float uses the single-precision bisection for
-// the airfoil.  Mesh links are found for a whole node at once by
-// mesh_links_warp.
+// Fraction q of the link of boundary node (x, y, z) towards the solid node x -
+// c at which the wall is crossed (wall point x_w = x - q c, q in (0,1]), and for
+// the walls their velocity (a sphere or airfoil moves with U, WallMotion).  R is
+// the collision arithmetic: double keeps the plain double evaluation; float
+// finds the airfoil's crossing in single precision.  Mesh links are found for a
+// whole node at once by mesh_links_warp.
+// what a block's boundary nodes share of the body's motion, in shared memory:
+// the velocity of a sphere or airfoil (and what is left of it in FP32) and the
+// airfoil's chord frame, converted and divided once a block, not once a node, on
+// the two FP64 lanes
+template <typename R>
+struct WallMotion {
+    R U[3];
+    float lo[3];
+    AirfoilFrame air;
+    // all threads of the block, 32 at least
+    __device__ __forceinline__ void load(const GeomParams &G, const DevBody *b)
+    {
+        const int t = threadIdx.x;
+        if (t < 3) {
+            const double u = b->U[t];
+            U[t] = (R)u;
+            lo[t] = (float)(u - (double)(R)u);
+        }
+        if (G.kind == LBM_BODY_AIRFOIL) {
+            if (t == 0) air.origin(G, b);
+            if (t < Q) air.direction(G, t);
+        }
+        __syncthreads();
+    }
+};
+
 template <typename R>
 __device__ __forceinline__ void link_data(const Lattice &L, const GeomParams &G, const DevBody *b,
-                                          int x, int y, int z, int cx, int cy, int cz, double &q,
-                                          double uw[3])
+                                          const AirfoilFrame &A, int x, int y, int z, int i, double &q,
+                                          R uw[3], float ul[3])
 {
-    constexpr bool single = sizeof(R) == 4;
-    if (G.kind == LBM_BODY_AIRFOIL && single) {
-        q = link_airfoil_f(G, b, x, y, cx, cy);
-        uw[0] = b->U[0];
-        uw[1] = b->U[1];
-        uw[2] = b->U[2];
+    const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+    if (G.kind == LBM_BODY_AIRFOIL && sizeof(R) == 4) {
+        q = link_airfoil_f(G, A, x, y, i);
     } else if (G.kind == LBM_BODY_SPHERE) {
         const double d0 = axis_offset(x, b->X[0], L.nx, G.periodic[0]);
         const double d1 = axis_offset(y, b->X[1], L.ny, G.periodic[1]);
@@ -586,9 +647,6 @@ __device__ __forceinline__ void link_data(const Lattice &L, const GeomParams &G,
         const double dd = d0 * d0 + d1 * d1 + d2 * d2;
         const double disc = cd * cd - cc * (dd - G.R * G.R);
         q = (cd - sqrt(fmax(disc, 0.0))) / cc;
-        uw[0] = b->U[0];
-        uw[1] = b->U[1];
-        uw[2] = b->U[2];
     } else if (G.kind == LBM_BODY_AIRFOIL) {
         // crossing of the link x - s c, s in [0, 1], by 50 bisections
         double lo = 0.0, hi = 1.0;
@@ -601,17 +659,15 @@ __device__ __forceinline__ void link_data(const Lattice &L, const GeomParams &G,
                 lo = mid;
         }
         q = 0.5 * (lo + hi);
-        uw[0] = b->U[0];
-        uw[1] = b->U[1];
-        uw[2] = b->U[2];
     } else {  // planes
         const double yb = (double)y;
         const bool low = (double)(y - cy) < G.y_lo;
         q = low ? (yb - G.y_lo) / (double)cy : (G.y_hi - yb) / (double)(-cy);
         const double *v = low ? G.U_lo : G.U_hi;
-        uw[0] = v[0];
-        uw[1] = v[1];
-        uw[2] = v[2];
+        for (int a = 0; a < 3; ++a) {
+            uw[a] = (R)v[a];
+            ul[a] = (float)(v[a] - (double)uw[a]);
+        }
     }
 }
 

@@ -195,36 +195,73 @@ __device__ __forceinline__ void fd_gradient(const R (*su)[4], const int *sok, co
 }
 
 // Stage populations of neighbourhood nodes selected by 'need' into sf[k][i]
-// and their density/velocity into su[k] (lane k).  sok[k] must be set.
-template <typename S, typename R>
+// and their density/velocity into su[k] (lane k).  sok[k] must be set.  The
+// nodes of a batch are loaded before any is stored, so that their latencies
+// overlap; one batch holds the nodes of a flat wall (itself, six neighbours,
+// eight more links).  (All 27 in line, most of them skipped, was a third of the
+// boundary kernel's instructions.)  ALL: all 27 at once, for a refilled node,
+// which needs most of them.
+template <typename S, typename R, bool ALL = false>
 __device__ __forceinline__ void stage(const Lattice &L, const S *__restrict__ fa, int lane, int nk,
                                       uint32_t need, R (*sf)[28], R (*su)[4], const int *sok)
 {
-    const size_t N = (size_t)L.N;
-    // all loads first, into registers, so they are in flight together (a
-    // store to shared memory right behind each load would wait out one
-    // memory latency per node)
-    R v[Q];
-    uint32_t got = 0;
+    constexpr int BATCH = 16;
+    const S *__restrict__ p = fa + (size_t)(lane < Q ? lane : 0) * (size_t)L.N;
+    if constexpr (ALL) {
+        R v[Q];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) {
-        const int nodek = __shfl_sync(FULL, nk, k);
-        const bool use = ((need >> k) & 1u) && nodek >= 0 && lane < Q;
-        v[k] = use ? Codec<S>::load(fa + (size_t)lane * N + nodek) : R(0);
-        got |= (use ? 1u : 0u) << k;
+        for (int k = 0; k < Q; ++k) {
+            const int node = __shfl_sync(FULL, nk, k);
+            v[k] = ((need >> k) & 1u) && node >= 0 && lane < Q ? Codec<S>::load(p + node) : R(0);
+        }
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+            if (lane < Q) sf[k][lane] = v[k];
     }
+    for (uint32_t m = ALL ? 0u : need; m;) {
+        R v[BATCH];
+        uint32_t t = m;
 #pragma unroll
-    for (int k = 0; k < Q; ++k)
-        if ((got >> k) & 1u) sf[k][lane] = v[k];
+        for (int j = 0; j < BATCH; ++j) {
+            v[j] = R(0);
+            if (t) {
+                const int node = __shfl_sync(FULL, nk, __ffs(t) - 1);
+                t &= t - 1;
+                if (node >= 0 && lane < Q) v[j] = Codec<S>::load(p + node);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j)
+            if (m) {
+                if (lane < Q) sf[__ffs(m) - 1][lane] = v[j];
+                m &= m - 1;
+            }
+    }
     __syncwarp();
     if (lane < Q && ((need >> lane) & 1u) && nk >= 0) {
+        R f[28];
+        if constexpr (sizeof(R) == 4) {
+            // (rows of 28 floats: eight lanes' quarter rows lie in different banks)
+#pragma unroll
+            for (int c = 0; c < 7; ++c) {
+                const float4 q = reinterpret_cast<const float4 *>(sf[lane])[c];
+                f[4 * c] = q.x;
+                f[4 * c + 1] = q.y;
+                f[4 * c + 2] = q.z;
+                f[4 * c + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) f[i] = sf[lane][i];
+        }
         R r = 0, j[3] = {0, 0, 0};
+#pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const R v = sf[lane][i];
-            r += v;
-            j[0] += R(cx_of(i)) * v;
-            j[1] += R(cy_of(i)) * v;
-            j[2] += R(cz_of(i)) * v;
+            const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
+            r += f[i];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                if (c[a]) j[a] = c[a] > 0 ? j[a] + f[i] : j[a] - f[i];
         }
         const R rho = R(L.rho0) + r;
         su[lane][0] = rho;
@@ -237,9 +274,64 @@ __device__ __forceinline__ void stage(const Lattice &L, const S *__restrict__ fa
 
 __device__ __forceinline__ void node_xyz(const Lattice &L, int n, int &x, int &y, int &z)
 {
-    x = n % L.nx;
-    y = (n / L.nx) % L.ny;
-    z = n / (L.nx * L.ny);
+    const int r = n / L.nx;
+    x = n - r * L.nx;
+    z = r / L.ny;
+    y = r - z * L.ny;
+}
+
+// offset of the neighbour along direction i away from the box faces
+__device__ __forceinline__ int direction_offset(const Lattice &L, int i)
+{
+    return cx_of(i) + L.nx * (cy_of(i) + L.ny * cz_of(i));
+}
+
+// neighbour x + c_i (-1 outside the box) and pull source x - c_i (-1 an
+// equilibrium face's value, -2 the bounce-back at a wall, which wins) of a node
+// on a box face; out of line, most bodies touch none
+__device__ __noinline__ static void face_sources(const Lattice &L, int x, int y, int z, int i, int &nk, int &src)
+{
+    const int c[3] = {cx_of(i), cy_of(i), cz_of(i)}, p0[3] = {x, y, z}, nn[3] = {L.nx, L.ny, L.nz};
+    int p[3], kind = 0;
+    for (int a = 0; a < 3; ++a) {
+        p[a] = p0[a] - c[a];
+        if (p[a] >= 0 && p[a] < nn[a]) continue;
+        const int face = L.face[2 * a + (p[a] < 0 ? 0 : 1)];
+        if (face == LBM_FACE_PERIODIC) p[a] = (p[a] + nn[a]) % nn[a];
+        else if (face == LBM_FACE_OUTFLOW) p[a] = p[a] < 0 ? 0 : nn[a] - 1;
+        else kind = max(kind, face == LBM_FACE_WALL ? 2 : 1);
+    }
+    src = kind ? -kind : p[0] + L.nx * (p[1] + L.ny * p[2]);
+    nk = neighbour(L, x, y, z, c[0], c[1], c[2]);
+}
+
+// Lane i < 27 of a boundary node: neighbour nk and pull source src along its
+// direction (face_sources), fluid marks of the neighbours into sok; returns the
+// missing set, the directions whose source is solid.  Off the faces sources and
+// neighbours are the same nodes, so one mark per lane gives both.  off:
+// direction_offset of the lane.
+__device__ __forceinline__ uint32_t node_links(const Lattice &L, const uint8_t *__restrict__ flags, int n, int x, int y,
+                                               int z, int lane, int off, int *sok, int &nk, int &src)
+{
+    const bool act = lane < Q;
+    nk = src = -1;
+    if (x > 0 && x < L.nx - 1 && y > 0 && y < L.ny - 1 && z > 0 && z < L.nz - 1) {
+        bool solid = false;
+        if (act) {
+            nk = n + off;
+            src = n - off;
+            solid = flags[nk] & FL_SOLID;
+            sok[lane] = !solid;
+        }
+        return __brev(__ballot_sync(FULL, solid && lane != 13)) >> (32 - Q);
+    }
+    bool solid = false;
+    if (act) {
+        face_sources(L, x, y, z, lane, nk, src);
+        sok[lane] = nk >= 0 && !(flags[nk] & FL_SOLID);
+        solid = lane != 13 && src >= 0 && (flags[src] & FL_SOLID);
+    }
+    return __ballot_sync(FULL, solid);
 }
 
 }  // namespace lbm
