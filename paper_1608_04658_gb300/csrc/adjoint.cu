@@ -27,6 +27,7 @@
 #include <cstring>
 
 #include "ctx.cuh"
+#include "kbcadj.cuh"
 #include "lanes.cuh"
 #include "pull.cuh"
 
@@ -69,178 +70,8 @@ __device__ __forceinline__ void axis_eq_adj(R u, R e[3], R phi[3], R r[3], R dl[
     dl[2] = D0 + dlnB;
 }
 
-// Transpose of the KBC collision f' = f - b (2 ds + g dh) (Eq. kbc_relax with
-// the analytic stabilizer), per node: lam holds dJ/df' on entry and dJ/df on
-// exit; g are the shifted pre-collision populations.  Backward sweep:
-//   ds_bar = -2b lam + a_bar dh/feq,  dh_bar = -b g lam + a_bar ds/feq + 2 b_bar dh/feq,
-//   g_bar = -b <lam, dh>,  a = <ds|dh>, b = <dh|dh>, g = 1/b - (2 - 1/b) a/b,
-//   df_bar = dh_bar + S^T (ds_bar - dh_bar),   feq_bar = -df_bar - (a_bar ds dh + b_bar dh^2)/feq^2,
-//   then f^eq(rho, u) and u = j/rho back to f.
-// Operation count as in the forward collision: moments from the x-lines of
-// the velocity cube, f^eq and 1/f^eq as products of per-axis factors with the
-// x-y pairs formed once, the shear values formed once.
-template <typename R>
-__device__ void kbc_vjp(const R g[Q], R lam[Q], R beta, R inv_beta, R rho0, int gamma_mode)
-{
-    R Ls[9], Ld[9];
-#pragma unroll
-    for (int l = 0; l < 9; ++l) {
-        Ld[l] = g[18 + l] - g[l];
-        Ls[l] = (g[18 + l] + g[l]) + g[9 + l];
-    }
-    const R drho = ((Ls[0] + Ls[1]) + (Ls[2] + Ls[3])) + ((Ls[4] + Ls[5]) + ((Ls[6] + Ls[7]) + Ls[8]));
-    const R jx = ((Ld[0] + Ld[1]) + (Ld[2] + Ld[3])) + ((Ld[4] + Ld[5]) + ((Ld[6] + Ld[7]) + Ld[8]));
-    const R jy = ((Ls[6] + Ls[7]) + Ls[8]) - ((Ls[0] + Ls[1]) + Ls[2]);
-    const R jz = ((Ls[2] + Ls[5]) + Ls[8]) - ((Ls[0] + Ls[3]) + Ls[6]);
-    const R rho = rho0 + drho, irho = rcp_fast(rho);
-    const R u[3] = {jx * irho, jy * irho, jz * irho};
-    R ex[3], ey[3], ez[3], px[3], py[3], pz[3], rx[3], ry[3], rz[3], dl[3][3];
-    axis_eq_adj(u[0], ex, px, rx, dl[0]);
-    axis_eq_adj(u[1], ey, py, ry, dl[1]);
-    axis_eq_adj(u[2], ez, pz, rz, dl[2]);
-    // f^eq_i = Fxy[cx][cy] Fz[cz], 1/f^eq_i = Rxy[cx][cy] Rz[cz] (1-D weights
-    // w(0) = 2/3, w(+-1) = 1/6 and rho folded in)
-    R Fxy[3][3], Rxy[3][3], Fz[3], Rz[3], exy[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const R w = a == 1 ? R(2.0 / 3.0) : R(1.0 / 6.0), iw = a == 1 ? R(1.5) : R(6);
-        Fz[a] = w * pz[a];
-        Rz[a] = iw * rz[a];
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const R wb = b == 1 ? R(2.0 / 3.0) : R(1.0 / 6.0), iwb = b == 1 ? R(1.5) : R(6);
-            Fxy[a][b] = rho * (w * px[a]) * (wb * py[b]);
-            Rxy[a][b] = irho * (iw * rx[a]) * (iwb * ry[b]);
-            exy[a][b] = ey[b] * px[a] + ex[a];
-        }
-    }
-    R rw[4], dw[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const R w = k == 0 ? R(8) / R(27) : k == 1 ? R(2) / R(27) : k == 2 ? R(1) / R(54) : R(1) / R(216);
-        rw[k] = rho * w;
-        dw[k] = drho * w;
-    }
-    R d[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i), nz = nonzero_of(i);
-        const R E = exy[cx + 1][cy + 1] * pz[cz + 1] + ez[cz + 1];
-        d[i] = g[i] - (rw[nz] * E + dw[nz]);
-    }
-    R A[9], B[9], T[9];
-#pragma unroll
-    for (int l = 0; l < 9; ++l) {
-        A[l] = d[18 + l] + d[l];
-        B[l] = d[18 + l] - d[l];
-        T[l] = A[l] + d[9 + l];
-    }
-    const R pxx = ((A[0] + A[1]) + (A[2] + A[3])) + ((A[4] + A[5]) + ((A[6] + A[7]) + A[8]));
-    const R pxy = ((B[6] + B[7]) + B[8]) - ((B[0] + B[1]) + B[2]);
-    const R pxz = ((B[2] + B[5]) + B[8]) - ((B[0] + B[3]) + B[6]);
-    const R pyy = ((T[0] + T[1]) + T[2]) + ((T[6] + T[7]) + T[8]);
-    const R pzz = ((T[0] + T[3]) + T[6]) + ((T[2] + T[5]) + T[8]);
-    const R pyz = (T[0] + T[8]) - (T[2] + T[6]);
-    const R nxz = pxx - pzz, nyz = pyy - pzz;
-    const R sx = (R(2) * nxz - nyz) * R(1.0 / 6.0);
-    const R sy = (R(2) * nyz - nxz) * R(1.0 / 6.0);
-    const R sz = -(nxz + nyz) * R(1.0 / 6.0);
-    const R qxy = R(0.25) * pxy, qxz = R(0.25) * pxz, qyz = R(0.25) * pyz;
-    R sh = 0, hh = 0, lh = 0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i), nz = nonzero_of(i);
-        const R ifeq = Rxy[cx + 1][cy + 1] * Rz[cz + 1];
-        if (nz == 1 || nz == 2) {
-            const R ds = shear_part<R>(i, sx, sy, sz, qxy, qxz, qyz);
-            const R dh = d[i] - ds;
-            const R t = dh * ifeq;
-            sh += ds * t;
-            hh += dh * t;
-            lh += lam[i] * dh;
-        } else {
-            hh += d[i] * (d[i] * ifeq);
-            lh += lam[i] * d[i];
-        }
-    }
-    const bool analytic = gamma_mode == LBM_GAMMA_ANALYTIC && hh > gamma_floor<R>();
-    const R ihh = analytic ? rcp_fast(hh) : R(0);
-    const R gam = analytic ? inv_beta - (R(2) - inv_beta) * sh * ihh : R(2);
-    const R gb = -beta * lh;
-    const R kk = R(2) - inv_beta;
-    const R ab = -kk * gb * ihh;
-    // (kk gb)(sh/hh)/hh: the square hh^2 would underflow in FP32 near rest
-    const R bb = kk * gb * (sh * ihh) * ihh;
-    const R cl_s = -R(2) * beta, cl_h = -beta * gam, bb2 = R(2) * bb;
-    // shear sums of ds_bar - dh_bar (faces and edges carry ds)
-    R Sx = 0, Sy = 0, Sz = 0, Qxy = 0, Qxz = 0, Qyz = 0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i), nz = nonzero_of(i);
-        if (nz != 1 && nz != 2) continue;
-        const R ifeq = Rxy[cx + 1][cy + 1] * Rz[cz + 1];
-        const R ds = shear_part<R>(i, sx, sy, sz, qxy, qxz, qyz);
-        const R dh = d[i] - ds;
-        // (ds_bar - dh_bar) = (cl_s - cl_h) lam + (ab (dh - ds) - 2 bb dh) / feq
-        const R t = (cl_s - cl_h) * lam[i] + (ab * (dh - ds) - bb2 * dh) * ifeq;
-        if (nz == 1) {
-            if (cx) Sx += t;
-            else if (cy) Sy += t;
-            else Sz += t;
-        } else {
-            if (cz == 0) Qxy += R(cx * cy) * t;
-            else if (cy == 0) Qxz += R(cx * cz) * t;
-            else Qyz += R(cy * cz) * t;
-        }
-    }
-    const R nxzb = (R(2) * Sx - Sy - Sz) * R(1.0 / 6.0);
-    const R nyzb = (R(2) * Sy - Sx - Sz) * R(1.0 / 6.0);
-    const R pzzb = -(nxzb + nyzb);
-    const R pxyb = R(0.25) * Qxy, pxzb = R(0.25) * Qxz, pyzb = R(0.25) * Qyz;
-    R rhob = 0, ub0 = 0, ub1 = 0, ub2 = 0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i), nz = nonzero_of(i);
-        const R ifeq = Rxy[cx + 1][cy + 1] * Rz[cz + 1];
-        const R feq = Fxy[cx + 1][cy + 1] * Fz[cz + 1];
-        // rest and corners carry no shear part (ds = 0, dh = d)
-        const bool sh_i = nz == 1 || nz == 2;
-        const R ds = sh_i ? shear_part<R>(i, sx, sy, sz, qxy, qxz, qyz) : R(0);
-        const R dh = sh_i ? d[i] - ds : d[i];
-        const R dhb = cl_h * lam[i] + (sh_i ? ab * ds + bb2 * dh : bb2 * dh) * ifeq;
-        // S^T of the shear sums: only the terms with nonzero c_a c_b (known
-        // per direction at compile time; a product with 0 would still cost an
-        // instruction)
-        R dfb = dhb;
-        if (cx) dfb += nxzb;
-        if (cy) dfb += nyzb;
-        if (cz) dfb += pzzb;
-        if (cx && cy) dfb = cx * cy > 0 ? dfb + pxyb : dfb - pxyb;
-        if (cx && cz) dfb = cx * cz > 0 ? dfb + pxzb : dfb - pxzb;
-        if (cy && cz) dfb = cy * cz > 0 ? dfb + pyzb : dfb - pyzb;
-        // feq_bar * feq
-        const R t = -(sh_i ? ab * ds + bb * dh : bb * dh) * dh * ifeq - dfb * feq;
-        rhob += t;
-        ub0 += t * dl[0][cx + 1];
-        ub1 += t * dl[1][cy + 1];
-        ub2 += t * dl[2][cz + 1];
-        lam[i] += dfb;
-    }
-    rhob *= irho;
-    const R jb[3] = {ub0 * irho, ub1 * irho, ub2 * irho};
-    rhob -= (ub0 * u[0] + ub1 * u[1] + ub2 * u[2]) * irho;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        R v = rhob;
-        if (cx_of(i)) v = cx_of(i) > 0 ? v + jb[0] : v - jb[0];
-        if (cy_of(i)) v = cy_of(i) > 0 ? v + jb[1] : v - jb[1];
-        if (cz_of(i)) v = cz_of(i) > 0 ? v + jb[2] : v - jb[2];
-        lam[i] += v;
-    }
-}
-
-// The same transpose with lane i < 27 holding g_i and lam_i (boundary nodes);
-// returns dJ/dg_i.
+// Transpose of the KBC collision (kbc_vjp_v) with lane i < 27 holding g_i and
+// lam_i (boundary nodes); returns dJ/dg_i.
 template <typename R>
 __device__ R kbc_vjp_lanes(R g, R lam, int i, R beta, R inv_beta, R rho0, int gamma_mode)
 {
@@ -417,29 +248,75 @@ __device__ __noinline__ R next_adjoint_rare(const Lattice &L, const GeomParams &
 }
 
 // lambda(S^{t+1})(x) of all directions: off the faces that need more, 27 plain
-// loads and the band's extra terms
+// loads and, where the node may lie in the band (near), its marks and extra terms
 template <typename R>
 __device__ __forceinline__ void next_adjoint_all(const Lattice &L, const GeomParams &G, const NextAdj<R> &A, int x,
-                                                 int y, int z, int n, R (&lam)[Q])
+                                                 int y, int z, int n, bool near, R (&lam)[Q])
 {
-    const size_t N = (size_t)L.N;
     int ox[3], oy[3], oz[3];
     bool special = axis_readers(x, L.nx, 1, L.face[0], L.face[1], ox);
     special |= axis_readers(y, L.ny, L.nx, L.face[2], L.face[3], oy);
     special |= axis_readers(z, L.nz, L.nx * L.ny, L.face[4], L.face[5], oz);
-    if (A.direct || special || (A.flags && (A.flags[n] & FL_UNCOVERED))) {
+    if (A.direct || special || (near && A.flags && (A.flags[n] & FL_UNCOVERED))) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) lam[i] = next_adjoint_rare<R>(L, G, A, x, y, z, n, i);
     } else {
         const R *p = A.lam + n;
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            lam[i] = p[(long long)i * (long long)N + (ox[cx_of(i) + 1] + oy[cy_of(i) + 1] + oz[cz_of(i) + 1])];
-        if (A.ext) {
+            lam[i] = p[L.plane[i] + (ox[cx_of(i) + 1] + oy[cy_of(i) + 1] + oz[cz_of(i) + 1])];
+        if (near && A.ext) {
             const int k = band_index(L, G, A.band, x, y, z);
             if (k >= 0) {
 #pragma unroll
                 for (int i = 0; i < Q; ++i) lam[i] += (R)A.ext[(size_t)k * Q + i];
+            }
+        }
+    }
+}
+
+// The same for the pair (x0, x0 + 1), x0 even: the aligned words of the pair, and
+// of its neighbours for c_x = +-1.
+__device__ __forceinline__ void next_adjoint_pair(const Lattice &L, const GeomParams &G, const NextAdj<float> &A, int x0,
+                                                  int y, int z, int n0, bool near, float2 (&lam)[Q])
+{
+    using P = Pair<float>;
+    int ox[3], oy[3], oz[3];
+    bool special = axis_readers(x0, L.nx, 1, L.face[0], L.face[1], ox);
+    special |= axis_readers(x0 + 1, L.nx, 1, L.face[0], L.face[1], ox);
+    special |= axis_readers(y, L.ny, L.nx, L.face[2], L.face[3], oy);
+    special |= axis_readers(z, L.nz, L.nx * L.ny, L.face[4], L.face[5], oz);
+    if (near && A.flags) special |= ((A.flags[n0] | A.flags[n0 + 1]) & FL_UNCOVERED) != 0;
+    if (A.direct) {
+        // (lambda_T is the caller's array: no more than its element's alignment)
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            lam[i] = A.lam ? make_float2(A.lam[n0 + L.plane[i]], A.lam[n0 + 1 + L.plane[i]]) : make_float2(0.f, 0.f);
+    } else if (special) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            lam[i] = make_float2(next_adjoint_rare<float>(L, G, A, x0, y, z, n0, i),
+                                 next_adjoint_rare<float>(L, G, A, x0 + 1, y, z, n0 + 1, i));
+    } else {
+        const int xl = x0 == 0 ? L.nx - 2 : -2, xr = x0 + 2 >= L.nx ? 2 - L.nx : 2;
+        const float *p = A.lam + n0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const int cx = cx_of(i);
+            const float *q = p + (L.plane[i] + oy[cy_of(i) + 1] + oz[cz_of(i) + 1]);
+            const float2 w = P::load(q);
+            if (cx == 0) lam[i] = w;
+            else if (cx > 0) lam[i] = P::cross(w, P::load(q + xr));  // readers x0 + 1, x0 + 2
+            else lam[i] = P::cross(P::load(q + xl), w);              // readers x0 - 1, x0
+        }
+        if (near && A.ext) {
+            const int ka = band_index(L, G, A.band, x0, y, z), kb = band_index(L, G, A.band, x0 + 1, y, z);
+            if (ka >= 0 || kb >= 0) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    if (ka >= 0) lam[i].x += (float)A.ext[(size_t)ka * Q + i];
+                    if (kb >= 0) lam[i].y += (float)A.ext[(size_t)kb * Q + i];
+                }
             }
         }
     }
@@ -460,7 +337,8 @@ __device__ __forceinline__ void next_adjoint_all(const Lattice &L, const GeomPar
 // no boundary node at t+1 and read neither; BAND the nodes of box0 that are
 // not in box1 (capacity-box grid).
 template <typename S>
-__global__ void __launch_bounds__(128, LBM_ADJ_MIN_BLOCKS) adjoint_bulk_kernel(const Lattice L, const GeomParams G,
+__global__ void __launch_bounds__(128, LBM_ADJ_MIN_BLOCKS) adjoint_bulk_kernel(const __grid_constant__ Lattice L,
+                                                           const __grid_constant__ GeomParams G,
                                                            const S *__restrict__ st,
                                                            const NextAdj<typename Codec<S>::R> A,
                                                            const uint8_t *__restrict__ flags1,
@@ -495,13 +373,100 @@ __global__ void __launch_bounds__(128, LBM_ADJ_MIN_BLOCKS) adjoint_bulk_kernel(c
         return;
     }
     if (f1 & FL_BOUNDARY) return;
+    // (outside box1 nothing of step t+1's band is read)
+    const bool near = mode != BULK_OUTSIDE || !box1;
     R lam[Q];
-    next_adjoint_all<R>(L, G, A, x, y, z, n, lam);
+    next_adjoint_all<R>(L, G, A, x, y, z, n, near, lam);
     R g[Q];
     gather_global<S>(L, st, x, y, z, n, g);
-    kbc_vjp<R>(g, lam, (R)L.beta, (R)L.inv_beta, (R)L.rho0, L.gamma_mode);
+    if constexpr (std::is_same<R, double>::value)
+        kbc_vjp_v<D1>(g, lam, L.beta, L.inv_beta, L.rho0, L.gamma_mode, (double)L.zero_f);
+    else
+        kbc_vjp_v<F1>(g, lam, L.beta_f, L.inv_beta_f, L.rho0_f, L.gamma_mode, L.zero_f);
+    R *q = lam_out + n;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) lam_out[(size_t)i * N + n] = lam[i];
+    for (int i = 0; i < Q; ++i) q[L.plane[i]] = lam[i];
+}
+
+// Two nodes per thread as in bulk_pair_kernel: ALL and OUTSIDE of FP32 and 16-bit
+// storage, rows of even length (an odd one's pairs are no aligned words).  PER:
+// all faces are periodic.  The 108 values of a pair's state and adjoint take 254
+// registers, 8 warps an SM, none spilled; with 90 loads of a warp in flight before
+// the first is used they cover the memory's latency.  324 bytes a node:
+// 256x128x128 FP32 341 us one node a thread (1870 instructions a node, 4.0 TB/s),
+// 238 us so (5.7 TB/s); at 168 registers the spill is 500 bytes.
+#ifndef LBM_ADJ_PAIR_MIN_BLOCKS
+#define LBM_ADJ_PAIR_MIN_BLOCKS 8
+#endif
+constexpr int ADJ_PAIR_THREADS = 32;
+template <typename S, bool PER>
+__global__ void __launch_bounds__(ADJ_PAIR_THREADS, LBM_ADJ_PAIR_MIN_BLOCKS) adjoint_pair_kernel(
+    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const S *__restrict__ st,
+    const __grid_constant__ NextAdj<float> A, const uint8_t *__restrict__ flags1, float *__restrict__ lam_out, int mode,
+    const int *__restrict__ box0, const int *__restrict__ box1)
+{
+    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x), y = blockIdx.y, z = blockIdx.z;
+    if (x0 >= L.nx) return;
+    int act = 3;  // bit 0: node x0 is updated here, bit 1: node x0 + 1
+    if (mode == BULK_OUTSIDE) {
+        const bool per = L.face[0] == LBM_FACE_PERIODIC;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int *box = k ? box1 : box0;
+            if (box && in_sweep(box, 1, y, L.ny, L.face[2] == LBM_FACE_PERIODIC) &&
+                in_sweep(box, 2, z, L.nz, L.face[4] == LBM_FACE_PERIODIC))
+                act &= (in_sweep(box, 0, x0, L.nx, per) ? 0 : 1) | (in_sweep(box, 0, x0 + 1, L.nx, per) ? 0 : 2);
+        }
+        if (!act) return;
+    }
+    const int n0 = x0 + L.nx * (y + L.ny * z);
+    float *q = lam_out + n0;
+    if (flags1) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint8_t f = flags1[n0 + k];
+            if ((act >> k & 1) && (f & FL_SOLID)) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) q[k + L.plane[i]] = 0.f;
+            }
+            if (f & (FL_SOLID | FL_BOUNDARY)) act &= ~(1 << k);
+        }
+        if (!act) return;
+    }
+    float2 lam[Q], g[Q];
+    next_adjoint_pair(L, G, A, x0, y, z, n0, mode != BULK_OUTSIDE || !box1, lam);
+    gather_pair<S, PER, PER, false>(L, st, x0, y, z, n0, g);
+    kbc_vjp_v<F2>(g, lam, L.beta_f, L.inv_beta_f, L.rho0_f, L.gamma_mode, L.zero_f);
+    if (act == 3) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) Pair<float>::store(q + L.plane[i], lam[i]);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        if (act & 1) q[L.plane[i]] = lam[i].x;
+        if (act & 2) q[1 + L.plane[i]] = lam[i].y;
+    }
+}
+
+// the bulk adjoint over the whole box (ALL, OUTSIDE)
+template <typename S>
+cudaError_t launch_adjoint_box(const Lattice &L, const GeomParams &G, const S *st, const NextAdj<typename Codec<S>::R> &A,
+                               const uint8_t *flags1, typename Codec<S>::R *lam_out, int mode, const int *box0,
+                               const int *box1, cudaStream_t s)
+{
+    if constexpr (!std::is_same<S, double>::value) {
+        if (L.nx % 2 == 0) {
+            const bool per = L.face[0] == LBM_FACE_PERIODIC && L.face[2] == LBM_FACE_PERIODIC && L.face[4] == LBM_FACE_PERIODIC;
+            auto kernel = per ? adjoint_pair_kernel<S, true> : adjoint_pair_kernel<S, false>;
+            const dim3 grid((L.nx / 2 + ADJ_PAIR_THREADS - 1) / ADJ_PAIR_THREADS, L.ny, L.nz);
+            kernel<<<grid, ADJ_PAIR_THREADS, 0, s>>>(L, G, st, A, flags1, lam_out, mode, box0, box1);
+            return cudaGetLastError();
+        }
+    }
+    const int bx = L.nx >= 128 ? 128 : ((L.nx + 31) / 32) * 32;
+    adjoint_bulk_kernel<S><<<dim3((L.nx + bx - 1) / bx, L.ny, L.nz), bx, 0, s>>>(L, G, st, A, flags1, lam_out, mode, box0, box1);
+    return cudaGetLastError();
 }
 
 // ----------------------------------------------------------------- centre-of-mass frame
@@ -730,10 +695,18 @@ struct BodyAdjoint {
 // refilled node there (6..11)
 constexpr int BODY_SLOTS = 12;
 
+// Resident blocks of the boundary adjoint asked of the register allocator: bound
+// by latency (2,000 instructions a node, issue 20 %), and its registers are taken
+// from the bulk adjoint beside it, so that 128 and a spill of 260 bytes beat 255
+// (256x128x128 swimmer, horizon 36: 41.1 ms for 41.9; 168 registers 41.4).  FP64
+// has its two lanes a clock to wait for.
+template <typename R>
+constexpr int LIST_ADJ_MIN_BLOCKS = sizeof(R) == 4 ? 4 : 1;
+
 // Boundary nodes of step t: forward recomputation of the Grad completion
 // (same operations as the boundary kernel), then its transpose.
 template <typename S>
-__global__ void __launch_bounds__(BWARPS * 32) adjoint_boundary_kernel(
+__global__ void __launch_bounds__(BWARPS * 32, LIST_ADJ_MIN_BLOCKS<typename Codec<S>::R>) adjoint_boundary_kernel(
     const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ blist,
     const int *__restrict__ bpos, const S *__restrict__ st, const NextAdj<typename Codec<S>::R> A,
     const uint8_t *__restrict__ flags1, typename Codec<S>::R *__restrict__ lam_out, double *__restrict__ ext,
@@ -1164,7 +1137,7 @@ __global__ void __launch_bounds__(128) lambda0_kernel(const Lattice L, const Geo
     if (x >= L.nx) return;
     const int n = x + L.nx * (y + L.ny * z);
     R lam[Q];
-    next_adjoint_all<R>(L, G, A, x, y, z, n, lam);
+    next_adjoint_all<R>(L, G, A, x, y, z, n, true, lam);
 #pragma unroll
     for (int i = 0; i < Q; ++i) out[(size_t)i * (size_t)L.N + n] = lam[i];
 }
@@ -1331,8 +1304,6 @@ cudaError_t reverse_step(lbm_ctx *ctx, const S *st, const NextAdj<typename Codec
     cudaStream_t s = ctx->stream;
     cudaStream_t side = ctx->side;
     cudaError_t e;
-    const int bx = L.nx >= 128 ? 128 : ((L.nx + 31) / 32) * 32;
-    dim3 grid((L.nx + bx - 1) / bx, L.ny, L.nz);
     if (split) {
         // band of step t (stored with state t) and of step t+1 (A.band)
         const int *box0 = (const int *)((const char *)(Sc.body + 0) + offsetof(DevBody, sweep));
@@ -1353,7 +1324,7 @@ cudaError_t reverse_step(lbm_ctx *ctx, const S *st, const NextAdj<typename Codec
             L, G, b, Sc.ulist, Sc.upos, st, lam_out, flags1, ext, tslots, bslot, ct);
         if (bslot) body_reduce_kernel<<<1, 256, 0, side>>>(bslot, capv, badj, G, b, ct, wx, wy, wz);
         if ((e = cudaEventRecord(ctx->ev_join, side)) != cudaSuccess) return e;
-        adjoint_bulk_kernel<S><<<grid, bx, 0, s>>>(L, G, st, A, nullptr, lam_out, BULK_OUTSIDE, box0, box1);
+        if ((e = launch_adjoint_box<S>(L, G, st, A, nullptr, lam_out, BULK_OUTSIDE, box0, box1, s)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(s, ctx->ev_join, 0)) != cudaSuccess) return e;
         return cudaGetLastError();
     }
@@ -1368,8 +1339,9 @@ cudaError_t reverse_step(lbm_ctx *ctx, const S *st, const NextAdj<typename Codec
             L, G, b, Sc.blist, Sc.bpos, st, A, flags1, lam_out, ext, tslots, badj, bslot, ct);
         if ((e = cudaEventRecord(ctx->ev_join, side)) != cudaSuccess) return e;
     }
-    adjoint_bulk_kernel<S><<<grid, bx, 0, s>>>(L, G, st, A, ctx->has_body ? flags1 : nullptr, lam_out, BULK_ALL,
-                                               nullptr, nullptr);
+    if ((e = launch_adjoint_box<S>(L, G, st, A, ctx->has_body ? flags1 : nullptr, lam_out, BULK_ALL, nullptr, nullptr, s)) !=
+        cudaSuccess)
+        return e;
     if (ctx->has_body) {
         if ((e = cudaStreamWaitEvent(s, ctx->ev_join, 0)) != cudaSuccess) return e;
         adjoint_refill_kernel<S><<<list_blocks(G.cap_uncovered), BWARPS * 32, 0, s>>>(
