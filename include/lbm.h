@@ -390,9 +390,9 @@ LBM_API lbm_status lbm_profile_end(lbm_ctx *ctx, double *total_ms, int64_t *laun
  *
  * Memory: the forward states are kept by checkpoint-and-recompute: every
  * checkpoint_every steps (0: ceil(sqrt(horizon))) a state is kept, and each
- * segment is recomputed once during the reverse sweep; the call allocates
- * (ceil(horizon/K) + K + 3) state buffers of 27 N elements and frees them
- * before returning (LBM_ERR_OOM if they do not fit).
+ * segment but the last is recomputed once during the reverse sweep; the call
+ * allocates at most (ceil(horizon/K) + K + 1) state buffers of 27 N elements and
+ * frees them before returning (LBM_ERR_OOM if they do not fit).
  *
  * On return the context has advanced by horizon steps, exactly as
  * lbm_step(horizon) would have (the forces of those steps are in the body

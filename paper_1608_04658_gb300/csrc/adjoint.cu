@@ -1217,8 +1217,9 @@ struct AdjBuffers {
 };
 
 // one forward step from fa into fb with the context's body scratch and the
-// given marks (the launch sequences of lbm_step; the force reduction only for
-// a free body, whose next pose needs it)
+// given marks (the launch sequences of lbm_step; the force reduction only for a
+// free body, whose next pose needs it).  fb NULL: the geometry and the
+// refill only, all that a reversed step needs of its own.
 cudaError_t forward_step(lbm_ctx *ctx, void *fa, void *fb, uint8_t *flags)
 {
     int nl = 0;
@@ -1226,6 +1227,12 @@ cudaError_t forward_step(lbm_ctx *ctx, void *fa, void *fb, uint8_t *flags)
     const uint8_t *fl = ctx->has_body ? flags : nullptr;
     int cur = ctx->bcur;
     int *status = &ctx->S.body[cur].status;
+    if (!fb) {
+        if (!ctx->has_body) return cudaSuccess;
+        ctx->bcur = cur ^ 1;
+        if ((e = launch_geometry(ctx->L, ctx->G, ctx->S, cur, flags, ctx->stream, &nl)) != cudaSuccess) return e;
+        return launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, ctx->bcur, fa, flags, ctx->stream);
+    }
     if (ctx->has_body && sweep_ahead(ctx->G) && ctx->order != ORDER_SEQUENTIAL) {
         // split order, as in lbm_step: the nodes outside the sweep box beside
         // the body's geometry, refill, boundary nodes and the box's nodes
@@ -1450,7 +1457,10 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
     const int nparts = 1024;
     double Jt = 0.0;
 
-    if (!B.get(&ck, (size_t)nseg * state) || !B.get(&seg, (size_t)(K + 1) * state) ||
+    // a segment's states: its checkpoint, which its first step may overwrite, and
+    // one for each of its other steps (the state after it is not read)
+    const auto seg_state = [&](int sg, int j) { return j == 0 ? ck + (size_t)sg * state : seg + (size_t)(j - 1) * state; };
+    if (!B.get(&ck, (size_t)nseg * state) || (K > 1 && !B.get(&seg, (size_t)(K - 1) * state)) ||
         !B.get(&ckflags, (size_t)nseg * N) || !B.get(&segflags, (size_t)(K + 1) * N) || !B.get(&wf[0], N) ||
         !B.get(&wf[1], N) || !B.get(&wrec, N) || !B.get(&ckbody, nseg) || !B.get(&segbody, K + 1) ||
         !B.get(&adjbody, 2) ||
@@ -1504,7 +1514,7 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
     ADJ_CUDA(cudaStreamSynchronize(s), "sync");
     for (int a = 0; a < 3; ++a) F0[a] = hb.F_sum[a];
     for (int t = 0; t < T; ++t) {
-        if (t % K == 0) {
+        if (t % K == 0 && t / K < nseg - 1) {
             const int k = t / K;
             ADJ_CUDA(cudaMemcpyAsync(ck + (size_t)k * state, ctx->f[ctx->cur], state * sizeof(S),
                                      cudaMemcpyDeviceToDevice, s), "checkpoint");
@@ -1512,8 +1522,26 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
             ADJ_CUDA(cudaMemcpyAsync(ckbody + k, ctx->S.body + ctx->bcur, sizeof(DevBody), cudaMemcpyDeviceToDevice, s),
                      "checkpoint");
         }
+        const int j = t - (nseg - 1) * K;
+        if (j < 0) {
+            st = lbm_step(ctx, 1);
+            if (st != LBM_OK) goto done;
+            continue;
+        }
+        // the last segment is reversed next: its steps leave their geometry, marks
+        // and (refilled) states where the reverse sweep expects them, a copy each
+        // (0.13 ms for a 256x128x128 swimmer) in place of the step again (0.25)
+        if (j == 0) {
+            ADJ_CUDA(cudaMemcpyAsync(segflags, ctx->flags, N, cudaMemcpyDeviceToDevice, s), "seg flags");
+            ADJ_CUDA(cudaMemcpyAsync(segbody, ctx->S.body + ctx->bcur, sizeof(DevBody), cudaMemcpyDeviceToDevice, s), "seg body");
+        }
+        if (body) use_slot(ctx, slots[j]);
         st = lbm_step(ctx, 1);
         if (st != LBM_OK) goto done;
+        ADJ_CUDA(cudaMemcpyAsync(seg_state(nseg - 1, j), ctx->f[ctx->cur ^ 1], state * sizeof(S), cudaMemcpyDeviceToDevice, s),
+                 "seg state");
+        ADJ_CUDA(cudaMemcpyAsync(segflags + (size_t)(j + 1) * N, ctx->flags, N, cudaMemcpyDeviceToDevice, s), "seg flags");
+        ADJ_CUDA(cudaMemcpyAsync(segbody + j + 1, ctx->S.body + ctx->bcur, sizeof(DevBody), cudaMemcpyDeviceToDevice, s), "seg body");
     }
     ADJ_CUDA(cudaMemcpyAsync(&hb, ctx->S.body + ctx->bcur, sizeof(DevBody), cudaMemcpyDeviceToHost, s), "body read");
     ADJ_CUDA(cudaMemcpyAsync(savebody, ctx->S.body, 2 * sizeof(DevBody), cudaMemcpyDeviceToDevice, s), "body save");
@@ -1545,22 +1573,24 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
         for (int sg = nseg - 1; sg >= 0; --sg) {
             NvtxRange nvtx_seg("adjoint segment");  // its recompute and its reversed steps
             const int t0 = sg * K, t1 = std::min(T, t0 + K);
-            // recompute the segment: seg[j] holds St^{t0+j} once step t0+j has run
-            ADJ_CUDA(cudaMemcpyAsync(seg, ck + (size_t)sg * state, state * sizeof(S), cudaMemcpyDeviceToDevice, s),
-                     "restore");
-            ADJ_CUDA(cudaMemcpyAsync(wrec, ckflags + (size_t)sg * N, N, cudaMemcpyDeviceToDevice, s), "restore");
-            ctx->bcur = 0;
-            ADJ_CUDA(cudaMemcpyAsync(ctx->S.body, ckbody + sg, sizeof(DevBody), cudaMemcpyDeviceToDevice, s), "restore");
-            // segflags[j] / segbody[j]: marks and body state before step t0 + j,
-            // which are also those that step t0 + j - 1's geometry left
-            for (int t = t0; t <= t1; ++t) {
-                const int j = t - t0;
-                ADJ_CUDA(cudaMemcpyAsync(segflags + (size_t)j * N, wrec, N, cudaMemcpyDeviceToDevice, s), "seg flags");
-                ADJ_CUDA(cudaMemcpyAsync(segbody + j, ctx->S.body + ctx->bcur, sizeof(DevBody), cudaMemcpyDeviceToDevice,
-                                         s), "seg body");
-                if (t == t1) break;
-                if (body) use_slot(ctx, slots[j]);
-                ADJ_CUDA(forward_step(ctx, seg + (size_t)j * state, seg + (size_t)(j + 1) * state, wrec), "recompute");
+            // recompute the segment from its checkpoint: seg_state(sg, j) holds
+            // St^{t0+j} once step t0+j has run.  segflags[j] / segbody[j]: marks and
+            // body state before step t0 + j, which are also those that step t0 + j -
+            // 1's geometry left
+            if (sg < nseg - 1) {
+                ADJ_CUDA(cudaMemcpyAsync(wrec, ckflags + (size_t)sg * N, N, cudaMemcpyDeviceToDevice, s), "restore");
+                ctx->bcur = 0;
+                ADJ_CUDA(cudaMemcpyAsync(ctx->S.body, ckbody + sg, sizeof(DevBody), cudaMemcpyDeviceToDevice, s), "restore");
+                for (int t = t0; t <= t1; ++t) {
+                    const int j = t - t0;
+                    ADJ_CUDA(cudaMemcpyAsync(segflags + (size_t)j * N, wrec, N, cudaMemcpyDeviceToDevice, s), "seg flags");
+                    ADJ_CUDA(cudaMemcpyAsync(segbody + j, ctx->S.body + ctx->bcur, sizeof(DevBody), cudaMemcpyDeviceToDevice, s),
+                             "seg body");
+                    if (t == t1) break;
+                    if (body) use_slot(ctx, slots[j]);
+                    ADJ_CUDA(forward_step(ctx, seg_state(sg, j), t + 1 < t1 ? seg_state(sg, j + 1) : nullptr, wrec),
+                             "recompute");
+                }
             }
             // the vertex tangents of every step of the segment at once, at the
             // pose each step's geometry left (segbody[j + 1])
@@ -1592,7 +1622,7 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
                     A = NextAdj<R>{lam[p ^ 1], body ? ext[p ^ 1] : nullptr, adjbody + (p ^ 1),
                                    body ? wf[p ^ 1] : nullptr, 0};
                 }
-                ADJ_CUDA(reverse_step<S>(ctx, seg + (size_t)j * state, A, wf[p], lam[p], ext[p], tslots, badj, bslot,
+                ADJ_CUDA(reverse_step<S>(ctx, seg_state(sg, j), A, wf[p], lam[p], ext[p], tslots, badj, bslot,
                                          badj0.fw[0], badj0.fw[1], badj0.fw[2], ct, cpart, cticket, split),
                          "reverse step");
                 if (body)
