@@ -1240,18 +1240,24 @@ cudaError_t forward_step(lbm_ctx *ctx, void *fa, void *fb, uint8_t *flags)
         cur = prev ^ 1;
         status = &ctx->S.body[cur].status;
         const int *sweep = ctx->S.body[prev].sweep;
+        const bool band_main = ctx->L.short_bulk;
+        const auto band = [&](cudaStream_t on) {
+            return launch_bulk(ctx->storage, ctx->L, fa, fb, flags, status, on, BULK_BAND, sweep, ctx->G.cap);
+        };
         if ((e = cudaEventRecord(ctx->ev_fork, ctx->stream)) != cudaSuccess ||
             (e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0)) != cudaSuccess ||
             (e = launch_geometry(ctx->L, ctx->G, ctx->S, prev, flags, ctx->side, &nl)) != cudaSuccess ||
             (e = launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, flags, ctx->side)) != cudaSuccess ||
+            (band_main && (e = cudaEventRecord(ctx->ev_marks, ctx->side)) != cudaSuccess) ||
             (e = launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, flags, ctx->side)) !=
                 cudaSuccess ||
             (ctx->G.free_motion && (e = launch_forces(ctx->storage, ctx->L, ctx->G, ctx->S, cur, flags, ctx->side, &nl)) != cudaSuccess) ||
-            (e = launch_bulk(ctx->storage, ctx->L, fa, fb, flags, status, ctx->side, BULK_BAND, sweep, ctx->G.cap)) !=
-                cudaSuccess ||
+            (!band_main && (e = band(ctx->side)) != cudaSuccess) ||
             (e = cudaEventRecord(ctx->ev_join, ctx->side)) != cudaSuccess ||
             (e = launch_bulk(ctx->storage, ctx->L, fa, fb, nullptr, status, ctx->stream, BULK_OUTSIDE, sweep)) !=
                 cudaSuccess ||
+            (band_main && ((e = cudaStreamWaitEvent(ctx->stream, ctx->ev_marks, 0)) != cudaSuccess ||
+                           (e = band(ctx->stream)) != cudaSuccess)) ||
             (e = cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0)) != cudaSuccess)
             return e;
         ctx->bcur = cur;

@@ -140,6 +140,7 @@ lbm_status lbm_create(const lbm_params *p, void *f_a, void *f_b, uint8_t *flags,
     L.inv_beta_f = (float)L.inv_beta;
     L.rho0_f = (float)L.rho0;
     L.zero_f = 0.0f;
+    L.short_bulk = 54 * (long long)elem_size(p->storage) * N < (1LL << 27);
     for (int i = 0; i < Q; ++i) L.g_face_f[i] = (float)L.g_face[i];
     ctx->storage = p->storage;
     ctx->elem = es;
@@ -162,12 +163,14 @@ lbm_status lbm_create(const lbm_params *p, void *f_a, void *f_b, uint8_t *flags,
     for (cudaEvent_t &e : ctx->ev_trial) trial_ok = trial_ok && cudaEventCreate(&e) == cudaSuccess;
     if (!trial_ok || cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, prio_greatest) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_marks, cudaEventDisableTiming) != cudaSuccess) {
         free_scratch(ctx, false);
         cudaFree(ctx->tot_partials);
         if (ctx->side) cudaStreamDestroy(ctx->side);
         if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
         if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+        if (ctx->ev_marks) cudaEventDestroy(ctx->ev_marks);
         for (cudaEvent_t e : ctx->ev_trial)
             if (e) cudaEventDestroy(e);
         delete ctx;
@@ -200,6 +203,7 @@ void lbm_destroy(lbm_ctx *ctx)
     for (cudaEvent_t e : ctx->prof) cudaEventDestroy(e);
     cudaEventDestroy(ctx->ev_fork);
     cudaEventDestroy(ctx->ev_join);
+    cudaEventDestroy(ctx->ev_marks);
     for (cudaEvent_t e : ctx->ev_trial) cudaEventDestroy(e);
     cudaStreamDestroy(ctx->side);
     if (ctx->copy) {
@@ -674,7 +678,9 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
         // geometry, refill, boundary nodes, force and the band's bulk nodes on
         // the side stream beside them; sequential, the geometry and refill run
         // first and the boundary nodes beside one flag-aware bulk launch.  The
-        // results are the same; the trial steps time both.
+        // results are the same; the trial steps time both.  Where the chain is the
+        // step (short_bulk), the band's bulk nodes follow those outside it on the
+        // caller's stream, once the marks and the refill are there.
         const bool ahead = ctx->has_body && sweep_ahead(ctx->G);
         bool split = ahead && ctx->order != ORDER_SEQUENTIAL;
         const bool trial = ahead && ctx->order == ORDER_UNDECIDED && ctx->trial < TRIAL_STEPS;
@@ -692,15 +698,23 @@ lbm_status lbm_step(lbm_ctx *ctx, int nsteps)
             LBM_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0), "fork wait");
             LBM_CUDA(launch_geometry(ctx->L, ctx->G, ctx->S, prev, ctx->flags, ctx->side, &launches), "geometry");
             LBM_CUDA(launch_refill(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, ctx->flags, ctx->side), "refill");
+            const bool band_main = ctx->L.short_bulk;
+            if (band_main) LBM_CUDA(cudaEventRecord(ctx->ev_marks, ctx->side), "marks");
             LBM_CUDA(launch_boundary(ctx->storage, ctx->L, ctx->G, ctx->S, cur, fa, fb, ctx->flags, ctx->side), "boundary");
             LBM_CUDA(launch_forces(ctx->storage, ctx->L, ctx->G, ctx->S, cur, ctx->flags, ctx->side, &launches), "forces");
-            LBM_CUDA(launch_bulk(ctx->storage, ctx->L, fa, fb, ctx->flags, status, ctx->side, BULK_BAND, sweep,
-                                 ctx->G.cap), "bulk band");
+            const auto band = [&](cudaStream_t on) {
+                return launch_bulk(ctx->storage, ctx->L, fa, fb, ctx->flags, status, on, BULK_BAND, sweep, ctx->G.cap);
+            };
+            if (!band_main) LBM_CUDA(band(ctx->side), "bulk band");
             LBM_CUDA(cudaEventRecord(ctx->ev_join, ctx->side), "join");
             LBM_CUDA(prof_mark(ctx, 0), "profile event");
             LBM_CUDA(launch_bulk(ctx->storage, ctx->L, fa, fb, nullptr, status, ctx->stream, BULK_OUTSIDE, sweep),
                      "bulk outside");
             LBM_CUDA(prof_mark(ctx, 1), "profile event");
+            if (band_main) {
+                LBM_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_marks, 0), "marks wait");
+                LBM_CUDA(band(ctx->stream), "bulk band");
+            }
             LBM_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0), "join wait");
             launches += 4;
         } else {

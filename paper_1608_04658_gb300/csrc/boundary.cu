@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
     const int *__restrict__ bpos, double *__restrict__ bforce, const S *__restrict__ fa,
     S *__restrict__ fb, const uint8_t *__restrict__ flags)
 {
+    after_previous();
     using R = typename Codec<S>::R;
     __shared__ __align__(16) R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
@@ -237,6 +238,7 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) refill_kerne
     const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ ulist,
     S *__restrict__ fa, const uint8_t *__restrict__ flags)
 {
+    after_previous();
     using R = typename Codec<S>::R;
     __shared__ __align__(16) R s_f[BWARPS][Q][28];
     __shared__ R s_u[BWARPS][Q][4];
@@ -312,9 +314,8 @@ cudaError_t launch_boundary(int storage, const Lattice &L, const GeomParams &G, 
     return dispatch_storage(storage, [&](auto tag) {
         using T = std::remove_pointer_t<decltype(tag)>;
         const int nb = list_blocks(G.cap_boundary, G.kind == LBM_BODY_MESH || G.kind == LBM_BODY_AIRFOIL ? LBM_LINK_LIST_BLOCKS : LBM_LIST_BLOCKS);
-        boundary_kernel<T><<<nb, BWARPS * 32, 0, s>>>(L, G, S.body + cur, S.blist, S.bpos, S.bforce, (const T *)fa,
-                                                      (T *)fb, flags);
-        return cudaGetLastError();
+        return launch_after(L.short_bulk, boundary_kernel<T>, nb, BWARPS * 32, s, L, G, S.body + cur, S.blist, S.bpos, S.bforce, (const T *)fa,
+                            (T *)fb, flags);
     });
 }
 
@@ -323,9 +324,8 @@ cudaError_t launch_refill(int storage, const Lattice &L, const GeomParams &G, Sc
 {
     return dispatch_storage(storage, [&](auto tag) {
         using T = std::remove_pointer_t<decltype(tag)>;
-        refill_kernel<T><<<list_blocks(G.cap_uncovered), BWARPS * 32, 0, s>>>(L, G, S.body + cur, S.ulist,
-                                                                               (T *)fa, flags);
-        return cudaGetLastError();
+        return launch_after(L.short_bulk, refill_kernel<T>, list_blocks(G.cap_uncovered), BWARPS * 32, s, L, G, S.body + cur, S.ulist, (T *)fa,
+                            flags);
     });
 }
 

@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(128, (BulkBlocks<S, FORM>::value)) bulk_kernel
                                                    const int *__restrict__ sweep, int mode, int capx,
                                                    int capy, int z0)
 {
+    after_previous();
     using R = typename Codec<S>::R;
     int x, y, z;
     if (mode == BULK_BAND) {
@@ -188,6 +189,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, PairBlocks<FORM>::value) bulk_pa
     const __grid_constant__ Lattice L, const S *__restrict__ fa, S *__restrict__ fb,
     const uint8_t *__restrict__ flags, int *__restrict__ status, const int *__restrict__ sweep, int mode, int z0)
 {
+    after_previous();
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x0 >= L.nx) return;
     const int y = blockIdx.y, z = z0 + (int)blockIdx.z;
@@ -207,6 +209,10 @@ template <typename S, int FORM>
 cudaError_t launch_bulk_form(const Lattice &L, const S *fa, S *fb, const uint8_t *flags, int *status, cudaStream_t s,
                              int mode, const int *sweep, const int *cap, int z_lo, int z_n)
 {
+    // early where no body's chain runs beside it or that chain is the step: the
+    // sweep box's blocks, waiting in their places at the end of a long chain, cost
+    // the bulk launch beside it half a percent
+    const bool early = (mode == BULK_ALL && !flags) || L.short_bulk;
     // FP32 and 16-bit storage take the two-node kernel for everything but the
     // sweep box (every node gets the same bits either way).  FP32 rows of odd
     // length stay with the one-node kernel, whose whole lines suit a launch bound
@@ -229,8 +235,7 @@ cudaError_t launch_bulk_form(const Lattice &L, const S *fa, S *fb, const uint8_t
                 else if (!odd && yzper) kernel = bulk_pair_kernel<S, FORM, false, true, false>;
             }
             const dim3 g2(((L.nx + 1) / 2 + PAIR_THREADS - 1) / PAIR_THREADS, L.ny, z_n);
-            kernel<<<g2, PAIR_THREADS, 0, s>>>(L, fa, fb, flags, status, sweep, mode, z_lo);
-            return cudaGetLastError();
+            return launch_after(early, kernel, g2, PAIR_THREADS, s, L, fa, fb, flags, status, sweep, mode, z_lo);
         }
     }
     int bx = L.nx >= 128 ? 128 : ((L.nx + 31) / 32) * 32;
@@ -243,8 +248,7 @@ cudaError_t launch_bulk_form(const Lattice &L, const S *fa, S *fb, const uint8_t
         const long long vol = (long long)cap[0] * cap[1] * cap[2];
         grid = dim3((unsigned)((vol + bx - 1) / bx), 1, 1);
     }
-    bulk_kernel<S, FORM><<<grid, bx, 0, s>>>(L, fa, fb, flags, status, sweep, mode, capx, capy, z_lo);
-    return cudaGetLastError();
+    return launch_after(early, bulk_kernel<S, FORM>, grid, bx, s, L, fa, fb, flags, status, sweep, mode, capx, capy, z_lo);
 }
 
 // FP32 and 16-bit boxes with a body and fewer nodes than this keep

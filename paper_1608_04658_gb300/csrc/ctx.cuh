@@ -29,7 +29,7 @@ struct lbm_ctx {
     lbm::Scratch S{};
     int bcur = 0;                 // body copy holding the latest state
     cudaStream_t side = nullptr;  // boundary + force kernels, overlapping the bulk kernel
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_marks = nullptr;
     double *plane = nullptr;      // N doubles for the host codec
     double *tot_partials = nullptr;
     int tot_blocks = 608;

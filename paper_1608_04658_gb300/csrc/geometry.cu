@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(GEOM_THREADS) mark_kernel(const Lattice L, con
                                                             DevBody *__restrict__ cur,
                                                             uint8_t *__restrict__ flags)
 {
+    after_previous();
     __shared__ double sX[3];
     __shared__ int slo[3], scnt[3];
     if (threadIdx.x == 0) {
@@ -277,6 +278,7 @@ __global__ void __launch_bounds__(GEOM_THREADS) classify_kernel(const Lattice L,
                                                                 int *__restrict__ ulist,
                                                                 int *__restrict__ upos)
 {
+    after_previous();
     const int cap = G.cap[0] * G.cap[1] * G.cap[2];
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -360,6 +362,7 @@ __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, c
                                                               double *__restrict__ partials,
                                                               unsigned *__restrict__ ticket)
 {
+    after_previous();
     const int cap = G.cap[0] * G.cap[1] * G.cap[2];
     const int chunk = (cap + gridDim.x - 1) / gridDim.x;
     const int beg = blockIdx.x * chunk;
@@ -461,6 +464,7 @@ __global__ void __launch_bounds__(POSE_THREADS) mesh_pose_kernel(const Lattice L
                                                                  DevBody *__restrict__ next, int advance,
                                                                  int ncols, int ncells)
 {
+    after_previous();
     __shared__ double sX[3], sU[3];
     if (threadIdx.x == 0) {
         double X[3], U[3];
@@ -529,6 +533,7 @@ __global__ void __launch_bounds__(POSE_THREADS) mesh_bin_kernel(const Lattice L,
                                                                 const DevBody *__restrict__ prev,
                                                                 const DevBody *__restrict__ next, int advance)
 {
+    after_previous();
     __shared__ int slo[3], scnt[3];
     if (threadIdx.x == 0) {
         double X[3], U[3];
@@ -748,10 +753,10 @@ cudaError_t launch_geometry(const Lattice &L, const GeomParams &G, Scratch &S, i
         if (G.com_frame && (e = launch_mesh_body(L, G, S, prev, true, s, nlaunch)) != cudaSuccess) return e;
         if ((e = launch_mesh_prepare(L, G, S, prev, true, s, nlaunch)) != cudaSuccess) return e;
     }
-    mark_kernel<<<nb, GEOM_THREADS, 0, s>>>(L, G, bp, bc, flags);
-    classify_kernel<<<nb, GEOM_THREADS, 0, s>>>(L, G, bc, flags, S.blist, S.bpos, S.ulist, S.upos);
     *nlaunch += 2;
-    return cudaGetLastError();
+    cudaError_t e;
+    if ((e = launch_after(L.short_bulk, mark_kernel, nb, GEOM_THREADS, s, L, G, bp, bc, flags)) != cudaSuccess) return e;
+    return launch_after(L.short_bulk, classify_kernel, nb, GEOM_THREADS, s, L, G, bc, flags, S.blist, S.bpos, S.ulist, S.upos);
 }
 
 cudaError_t launch_mark_initial(const Lattice &L, const GeomParams &G, const double *X,
@@ -770,9 +775,8 @@ cudaError_t launch_forces(int storage, const Lattice &L, const GeomParams &G, Sc
     // and a round trip to memory (airfoil, 240,000 positions: 128 blocks 28 us)
     const long long cap = (long long)G.cap[0] * G.cap[1] * G.cap[2];
     const int nb = (int)std::min<long long>(S.n_partials, (cap + 2 * FORCE_THREADS - 1) / (2 * FORCE_THREADS));
-    kernel<<<nb, FORCE_THREADS, 0, s>>>(L, G, S.body + cur, flags, S.bforce, S.partials, S.ticket);
     *nlaunch += 1;
-    return cudaGetLastError();
+    return launch_after(L.short_bulk, kernel, nb, FORCE_THREADS, s, L, G, S.body + cur, flags, S.bforce, S.partials, S.ticket);
 }
 
 cudaError_t launch_sweep_init(const Lattice &L, const GeomParams &G, Scratch &S, int cur, cudaStream_t s)
@@ -796,9 +800,8 @@ cudaError_t launch_mesh_prepare(const Lattice &L, const GeomParams &G, Scratch &
     DevBody *next = S.body + (advance ? prev ^ 1 : prev);
     mesh_pose_kernel<<<nb_v > 0 ? nb_v : 1, POSE_THREADS, 0, s>>>(L, G, S.body + prev, next, advance ? 1 : 0, ncols,
                                                                     ncells);
-    mesh_bin_kernel<<<nb_t > 0 ? nb_t : 1, POSE_THREADS, 0, s>>>(L, G, S.body + prev, next, advance ? 1 : 0);
     *nlaunch += 2;
-    return cudaGetLastError();
+    return launch_after(L.short_bulk, mesh_bin_kernel, nb_t > 0 ? nb_t : 1, POSE_THREADS, s, L, G, S.body + prev, next, advance ? 1 : 0);
 }
 
 cudaError_t launch_mesh_mark_initial(const Lattice &L, const GeomParams &G, Scratch &S, int cur,

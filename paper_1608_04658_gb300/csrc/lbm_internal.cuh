@@ -89,6 +89,12 @@ struct Lattice {
     // bulk kernels (no FP64 conversion on the device)
     float beta_f, inv_beta_f, rho0_f;
     float g_face_f[27];
+    // The bulk launch moves less than 2^27 bytes (54 values a node; 20 us): the
+    // body's chain of 40 us and more is the step.  It launches early
+    // (launch_after) and the sweep box's nodes are not at its end (lbm_step).
+    // Measured: 99 MB sphere 790 -> 712 us, 164 MB airfoil 306 and 307, 806 MB
+    // airfoil 1100 -> 1160.
+    int short_bulk;
     float zero_f;       // 0, not known to the compiler (see kbc_collide_v)
 };
 
@@ -99,6 +105,34 @@ struct Lattice {
 // {lo x, lo y, lo z, n x, n y, n z} of the box, in device memory (wrapping on
 // periodic axes); cap = capacity of the box per axis (the BAND grid).
 enum BulkMode { BULK_ALL = 0, BULK_OUTSIDE = 1, BULK_BAND = 2 };
+
+// Programmatic dependent launch, for the kernels of a step, which follow each
+// other on a stream: launch_after lets a kernel's blocks take their places while
+// the previous one's last blocks still run, and after_previous, first in every
+// such kernel and in all its threads, waits until that kernel has completed and
+// its writes are seen (so the end of one implies the end of all before it), and
+// lets the next one's blocks in.  Without the attribute, or behind a copy or an
+// event, it is an ordinary launch.  (A step of a 32^3 box is a launch of 5 us,
+// most of it its start; the chain of a small body has six of them.)
+__device__ __forceinline__ void after_previous()
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... K, typename... A>
+cudaError_t launch_after(bool early, void (*kernel)(K...), dim3 grid, int threads, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<K>(args)...);
+}
 
 // Calls fn with a null pointer of the storage type (one instantiation per
 // storage form).
