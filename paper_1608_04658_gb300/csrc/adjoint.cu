@@ -960,7 +960,7 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_refill_kernel(
             const double *v = (double)y < 0.5 * (G.y_lo + G.y_hi) ? G.U_lo : G.U_hi;
             ud[0] = v[0]; ud[1] = v[1]; ud[2] = v[2];
         } else if (G.kind == LBM_BODY_MESH) {
-            mesh_material_velocity(G, b, (double)x, (double)y, ud);
+            mesh_material_velocity_warp(G, b, (double)x, (double)y, lane, ud);
         }
         const R u[3] = {(R)ud[0], (R)ud[1], (R)ud[2]};
         R du[3][3];
@@ -992,12 +992,17 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_refill_kernel(
                 if (d < 3) tb[d] = v;
                 else gb[d - 3] = v;
             }
-        } else if (lane == 0 && G.kind == LBM_BODY_MESH) {
-            double dv[3];
-            swimmer_velocity_tangent(G, b->t, clamp_arc(G, (double)x - b->X[0]), dv);
+        } else if (G.kind == LBM_BODY_MESH && !G.com_frame) {
+            // the tangents at t + 1 in the even lanes, at t - 1 in the odd ones, half
+            // their difference (swimmer_velocity_tangent, swimmer_rate_dX)
+            const double sr = (double)x - b->X[0], t1 = lane & 1 ? b->t - 1.0 : b->t + 1.0;
+            double dv[4];
+            swimmer_midline_tangent(G, clamp_arc(G, sr), t1, dv);
+            dv[3] = bslot && sr >= 0.0 && sr <= G.length ? -swimmer_midline_ds(G, sr, t1) : 0.0;
+            for (int k = 0; k < 4; ++k) dv[k] = 0.5 * (__shfl_sync(FULL, dv[k], 0) - __shfl_sync(FULL, dv[k], 1));
             for (int k = 0; k < 3; ++k) tb[k] = (double)ub[1] * dv[k];
             // the head frame: U0 e_x + rate(x - X0) e_y
-            gb[0] = (double)ub[1] * swimmer_rate_dX(G, b->t, (double)x - b->X[0]);
+            gb[0] = (double)ub[1] * dv[3];
             gb[3] = (double)ub[0];
         } else if (lane == 0 && G.kind == LBM_BODY_SPHERE) {
             for (int a = 0; a < 3; ++a) gb[3 + a] = (double)ub[a];  // the refill velocity is U

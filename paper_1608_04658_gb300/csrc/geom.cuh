@@ -178,6 +178,30 @@ __device__ __forceinline__ void mesh_material_velocity(const GeomParams &G, cons
     v[2] = b->U[2];
 }
 
+// The same by a warp, every lane with the same point: the midline at t + 1 in the
+// even lanes and at t - 1 in the odd ones, a sine and its divisions (FP64, some
+// 4 us of latency in the small refill kernels) once, not one after the other.
+__device__ __forceinline__ void mesh_material_velocity_warp(const GeomParams &G, const DevBody *b, double px, double py,
+                                                            int lane, double v[3])
+{
+    const double cs = G.com_frame ? cos(b->psi) : 1.0, sn = G.com_frame ? sin(b->psi) : 0.0;
+    const double rx = px - b->X[0], ry = py - b->X[1];
+    const double s = clamp_arc(G, G.com_frame ? cs * rx + sn * ry + b->com[0] : rx);
+    const double m = swimmer_midline(G, s, lane & 1 ? __dsub_rn(b->t, 1.0) : __dadd_rn(b->t, 1.0));
+    const double m1 = __shfl_sync(0xffffffffu, m, 0), m0 = __shfl_sync(0xffffffffu, m, 1);
+    const double rate = __ddiv_rn(__dsub_rn(m1, m0), 2.0);
+    if (!G.com_frame) {
+        v[0] = b->U[0];
+        v[1] = __dadd_rn(b->U[1], rate);
+        v[2] = b->U[2];
+        return;
+    }
+    const double wx = -b->com_dot[0], wy = rate - b->com_dot[1];
+    v[0] = b->U[0] - b->omega * ry + (cs * wx - sn * wy);
+    v[1] = b->U[1] + b->omega * rx + (sn * wx + cs * wy);
+    v[2] = b->U[2];
+}
+
 // edge value of the (y, z) projection of directed edge u -> v at (y, z),
 // evaluated from the lower-index vertex; sign with zero counted positive in
 // that direction
