@@ -19,6 +19,9 @@ namespace lbm {
 // or b_bar with it is a ratio).  d ln Phi(c)/du = D0 + c dlnB per axis, so the
 // velocity's adjoint needs four sums over the directions of t = feq_bar feq, as
 // the density's: sum t and sum c t.
+// Against 64 bits from the same state (48^3 box, FP32, lambda_T random): 3.5e-6
+// after eight steps where per-direction derivatives and absolute 1/f^eq gave
+// 4.2e-6, 6.4e-7 and 6.0e-7 after one.
 // zero: a run-time 0 (see kbc_collide_m).
 template <typename O>
 __device__ __forceinline__ void kbc_vjp_v(typename O::V (&g)[Q], typename O::V (&lam)[Q], typename O::R beta,
