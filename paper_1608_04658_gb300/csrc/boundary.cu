@@ -49,10 +49,10 @@ namespace lbm {
 // pipe of two lanes a clock and SM: it took the larger part of this kernel's
 // time (airfoil 225 us with it).  The force kernel does it for 32 nodes a warp.
 template <typename R>
-__device__ __forceinline__ void node_force(double *__restrict__ slot, int lane, bool link, int cx, int cy, int cz,
+__device__ __forceinline__ void node_force(double *slot, int lane, bool link, int cx, int cy, int cz,
                                            int i, R fbb, R gi, R q, const R uw[3], const float ul[3]);
 template <>
-__device__ __forceinline__ void node_force<double>(double *__restrict__ slot, int lane, bool link, int cx, int cy,
+__device__ __forceinline__ void node_force<double>(double *slot, int lane, bool link, int cx, int cy,
                                                    int cz, int i, double fbb, double gi, double q, const double uw[3],
                                                    const float ul[3])
 {
@@ -77,7 +77,7 @@ __device__ __forceinline__ void node_force<double>(double *__restrict__ slot, in
     if (lane == 0) reinterpret_cast<ForceSlot<double> *>(slot)->k = pack_k(k0, k1, k2);
 }
 template <>
-__device__ __forceinline__ void node_force<float>(double *__restrict__ slot, int lane, bool link, int cx, int cy,
+__device__ __forceinline__ void node_force<float>(double *slot, int lane, bool link, int cx, int cy,
                                                   int cz, int i, float fbb, float gi, float q, const float uw[3],
                                                   const float ul[3])
 {
@@ -127,9 +127,9 @@ __device__ __forceinline__ void node_force<float>(double *__restrict__ slot, int
 
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_kernel(
-    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, DevBody *__restrict__ b, const int *__restrict__ blist,
-    const int *__restrict__ bpos, double *__restrict__ bforce, const S *__restrict__ fa,
-    S *__restrict__ fb, const uint8_t *__restrict__ flags)
+    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, DevBody *b, const int *blist,
+    const int *bpos, double *bforce, const S *fa,
+    S *fb, const uint8_t *flags)
 {
     after_previous();
     using R = typename Codec<S>::R;
@@ -235,8 +235,8 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
 
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) refill_kernel(
-    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const DevBody *__restrict__ b, const int *__restrict__ ulist,
-    S *__restrict__ fa, const uint8_t *__restrict__ flags)
+    const __grid_constant__ Lattice L, const __grid_constant__ GeomParams G, const DevBody *b, const int *ulist,
+    S *fa, const uint8_t *flags)
 {
     after_previous();
     using R = typename Codec<S>::R;

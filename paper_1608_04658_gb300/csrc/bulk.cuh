@@ -51,8 +51,8 @@ constexpr int PAIR_THREADS = 32;
 // iteration, out of line and after everything else of its thread: the few nodes
 // that exact_stabilizer hands back.
 template <typename S>
-__device__ __noinline__ void exact_node_update(const Lattice &L, const S *__restrict__ fa, S *__restrict__ fb,
-                                               int *__restrict__ status, int x, int y, int z)
+__device__ __noinline__ void exact_node_update(const Lattice &L, const S *fa, S *fb,
+                                               int *status, int x, int y, int z)
 {
     using R = typename Codec<S>::R;
     const int n = x + L.nx * (y + L.ny * z);
@@ -64,11 +64,11 @@ __device__ __noinline__ void exact_node_update(const Lattice &L, const S *__rest
 }
 
 template <typename S, int FORM>
-__global__ void __launch_bounds__(128, (BulkBlocks<S, FORM>::value)) bulk_kernel(const __grid_constant__ Lattice L, const S *__restrict__ fa,
-                                                   S *__restrict__ fb,
-                                                   const uint8_t *__restrict__ flags,
-                                                   int *__restrict__ status,
-                                                   const int *__restrict__ sweep, int mode, int capx,
+__global__ void __launch_bounds__(128, (BulkBlocks<S, FORM>::value)) bulk_kernel(const __grid_constant__ Lattice L, const S *fa,
+                                                   S *fb,
+                                                   const uint8_t *flags,
+                                                   int *status,
+                                                   const int *sweep, int mode, int capx,
                                                    int capy, int z0)
 {
     after_previous();
@@ -130,9 +130,9 @@ __global__ void __launch_bounds__(128, (BulkBlocks<S, FORM>::value)) bulk_kernel
 // kernel), per node of the pair.  XPER: the x axis is periodic; YZPER: the y and
 // z axes are.
 template <typename S, int FORM, bool XPER, bool YZPER, bool ODD>
-__device__ __forceinline__ void pair_update(const Lattice &L, const S *__restrict__ fa, S *__restrict__ fb,
-                                            const uint8_t *__restrict__ flags, int *__restrict__ status,
-                                            const int *__restrict__ sweep, int mode, int x0, int y, int z)
+__device__ __forceinline__ void pair_update(const Lattice &L, const S *fa, S *fb,
+                                            const uint8_t *flags, int *status,
+                                            const int *sweep, int mode, int x0, int y, int z)
 {
     int act = 3;  // bit 0: node x0 is updated here, bit 1: node x0 + 1
     if (ODD && x0 + 1 == L.nx) {
@@ -186,8 +186,8 @@ __device__ __forceinline__ void pair_update(const Lattice &L, const S *__restric
 // faces are (the choice is uniform over the block).
 template <typename S, int FORM, bool XPER, bool YZPER, bool ODD>
 __global__ void __launch_bounds__(PAIR_THREADS, PairBlocks<FORM>::value) bulk_pair_kernel(
-    const __grid_constant__ Lattice L, const S *__restrict__ fa, S *__restrict__ fb,
-    const uint8_t *__restrict__ flags, int *__restrict__ status, const int *__restrict__ sweep, int mode, int z0)
+    const __grid_constant__ Lattice L, const S *fa, S *fb,
+    const uint8_t *flags, int *status, const int *sweep, int mode, int z0)
 {
     after_previous();
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);

@@ -205,7 +205,7 @@ __device__ __forceinline__ void mesh_material_velocity_warp(const GeomParams &G,
 // edge value of the (y, z) projection of directed edge u -> v at (y, z),
 // evaluated from the lower-index vertex; sign with zero counted positive in
 // that direction
-__device__ __forceinline__ double mesh_edge(const double *__restrict__ P, int u, int v, double y, double z, int &sg)
+__device__ __forceinline__ double mesh_edge(const double *P, int u, int v, double y, double z, int &sg)
 {
     const int a = u < v ? u : v, b = u < v ? v : u;
     const double Ay = P[3 * a + 1], Az = P[3 * a + 2], By = P[3 * b + 1], Bz = P[3 * b + 2];
@@ -216,7 +216,7 @@ __device__ __forceinline__ double mesh_edge(const double *__restrict__ P, int u,
 }
 
 // does the line {(., y, z)} cross triangle t?  xc = crossing abscissa
-__device__ __forceinline__ bool mesh_column_crossing(const double *__restrict__ P, int t0, int t1, int t2,
+__device__ __forceinline__ bool mesh_column_crossing(const double *P, int t0, int t1, int t2,
                                                      double y, double z, double &xc)
 {
     int s0, s1, s2;

@@ -204,9 +204,9 @@ __device__ __forceinline__ bool band_node(const Lattice &L, const GeomParams &G,
 }
 
 __global__ void __launch_bounds__(GEOM_THREADS) mark_kernel(const Lattice L, const GeomParams G,
-                                                            const DevBody *__restrict__ prev,
-                                                            DevBody *__restrict__ cur,
-                                                            uint8_t *__restrict__ flags)
+                                                            const DevBody *prev,
+                                                            DevBody *cur,
+                                                            uint8_t *flags)
 {
     after_previous();
     __shared__ double sX[3];
@@ -271,12 +271,12 @@ __global__ void __launch_bounds__(GEOM_THREADS) mark_kernel(const Lattice L, con
 }
 
 __global__ void __launch_bounds__(GEOM_THREADS) classify_kernel(const Lattice L, const GeomParams G,
-                                                                DevBody *__restrict__ cur,
-                                                                uint8_t *__restrict__ flags,
-                                                                int *__restrict__ blist,
-                                                                int *__restrict__ bpos,
-                                                                int *__restrict__ ulist,
-                                                                int *__restrict__ upos)
+                                                                DevBody *cur,
+                                                                uint8_t *flags,
+                                                                int *blist,
+                                                                int *bpos,
+                                                                int *ulist,
+                                                                int *upos)
 {
     after_previous();
     const int cap = G.cap[0] * G.cap[1] * G.cap[2];
@@ -356,11 +356,11 @@ __global__ void mark_initial_kernel(const Lattice L, const GeomParams G, const d
 // marks say which, one byte a node in place of clearing and reading 48)
 template <typename R>
 __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, const GeomParams G,
-                                                              DevBody *__restrict__ cur,
-                                                              const uint8_t *__restrict__ flags,
-                                                              const double *__restrict__ bforce,
-                                                              double *__restrict__ partials,
-                                                              unsigned *__restrict__ ticket)
+                                                              DevBody *cur,
+                                                              const uint8_t *flags,
+                                                              const double *bforce,
+                                                              double *partials,
+                                                              unsigned *ticket)
 {
     after_previous();
     const int cap = G.cap[0] * G.cap[1] * G.cap[2];
@@ -460,8 +460,8 @@ __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, c
 // frame) or X + R(psi) (b - c(t)) (centre-of-mass frame, with the lattice box
 // of the pose) and velocities; clears the column and cell lists of the step.
 __global__ void __launch_bounds__(POSE_THREADS) mesh_pose_kernel(const Lattice L, const GeomParams G,
-                                                                 const DevBody *__restrict__ prev,
-                                                                 DevBody *__restrict__ next, int advance,
+                                                                 const DevBody *prev,
+                                                                 DevBody *next, int advance,
                                                                  int ncols, int ncells)
 {
     after_previous();
@@ -530,8 +530,8 @@ __global__ void __launch_bounds__(POSE_THREADS) mesh_pose_kernel(const Lattice L
 // Per triangle: its box, the band columns whose line crosses it (with the
 // crossing abscissa) and the band cells its box overlaps.
 __global__ void __launch_bounds__(POSE_THREADS) mesh_bin_kernel(const Lattice L, const GeomParams G,
-                                                                const DevBody *__restrict__ prev,
-                                                                const DevBody *__restrict__ next, int advance)
+                                                                const DevBody *prev,
+                                                                const DevBody *next, int advance)
 {
     after_previous();
     __shared__ int slo[3], scnt[3];

@@ -202,11 +202,11 @@ __device__ __forceinline__ void fd_gradient(const R (*su)[4], const int *sok, co
 // boundary kernel's instructions.)  ALL: all 27 at once, for a refilled node,
 // which needs most of them.
 template <typename S, typename R, bool ALL = false>
-__device__ __forceinline__ void stage(const Lattice &L, const S *__restrict__ fa, int lane, int nk,
+__device__ __forceinline__ void stage(const Lattice &L, const S *fa, int lane, int nk,
                                       uint32_t need, R (*sf)[28], R (*su)[4], const int *sok)
 {
     constexpr int BATCH = 16;
-    const S *__restrict__ p = fa + (size_t)(lane < Q ? lane : 0) * (size_t)L.N;
+    const S *p = fa + (size_t)(lane < Q ? lane : 0) * (size_t)L.N;
     if constexpr (ALL) {
         R v[Q];
 #pragma unroll
@@ -310,7 +310,7 @@ __device__ __noinline__ static void face_sources(const Lattice &L, int x, int y,
 // missing set, the directions whose source is solid.  Off the faces sources and
 // neighbours are the same nodes, so one mark per lane gives both.  off:
 // direction_offset of the lane.
-__device__ __forceinline__ uint32_t node_links(const Lattice &L, const uint8_t *__restrict__ flags, int n, int x, int y,
+__device__ __forceinline__ uint32_t node_links(const Lattice &L, const uint8_t *flags, int n, int x, int y,
                                                int z, int lane, int off, int *sok, int &nk, int &src)
 {
     const bool act = lane < Q;

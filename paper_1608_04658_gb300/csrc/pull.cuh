@@ -38,7 +38,7 @@ __device__ __forceinline__ void axis_off(int a, int n, int stride, int face_lo, 
 
 // coordinate c on axis a (n nodes) inside the sweep box sw = {lo[3], n[3]}
 // (wrapping on a periodic axis, where lo lies in (-n, n))
-__device__ __forceinline__ bool in_sweep(const int *__restrict__ sw, int a, int c, int n, bool periodic)
+__device__ __forceinline__ bool in_sweep(const int *sw, int a, int c, int n, bool periodic)
 {
     int d = c - sw[a];
     if (periodic) {
@@ -48,7 +48,7 @@ __device__ __forceinline__ bool in_sweep(const int *__restrict__ sw, int a, int 
     return (unsigned)d < (unsigned)sw[3 + a];
 }
 
-__device__ __forceinline__ bool in_sweep_box(const Lattice &L, const int *__restrict__ sw, int x, int y, int z)
+__device__ __forceinline__ bool in_sweep_box(const Lattice &L, const int *sw, int x, int y, int z)
 {
     return in_sweep(sw, 1, y, L.ny, L.face[2] == LBM_FACE_PERIODIC) &&
            in_sweep(sw, 2, z, L.nz, L.face[4] == LBM_FACE_PERIODIC) &&
@@ -62,7 +62,7 @@ __device__ __forceinline__ int sweep_coord(int v, int n)
 
 // pulls of node (x, y, z) from global memory under the box rules
 template <typename S>
-__device__ __forceinline__ void gather_global(const Lattice &L, const S *__restrict__ fa, int x, int y, int z,
+__device__ __forceinline__ void gather_global(const Lattice &L, const S *fa, int x, int y, int z,
                                               int n, typename Codec<S>::R g[Q])
 {
     using R = typename Codec<S>::R;
@@ -153,7 +153,7 @@ template <> struct Pair<__nv_bfloat16> {
 //   (loaded then), an equilibrium face its value (not over an x wall's), and an
 //   equilibrium x face its value in the outer node (not over a y or z wall's).
 template <typename S, bool XPER, bool YZPER, bool ODD>
-__device__ __forceinline__ void gather_pair(const Lattice &L, const S *__restrict__ fa, int x0, int y, int z,
+__device__ __forceinline__ void gather_pair(const Lattice &L, const S *fa, int x0, int y, int z,
                                             int n0, float2 g[Q])
 {
     using P = Pair<S>;
