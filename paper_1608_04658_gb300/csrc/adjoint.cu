@@ -1652,8 +1652,10 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
         }
     }
     if (com && (ctx->G.free_motion & 4)) {
-        com_tangent_kernel<<<(ctx->G.n_triangles + 255) / 256, 256, 0, s>>>(ctx->G, ckbody, cpart, cticket, ct);
-        initial_spin_kernel<<<1, 32, 0, s>>>(badj, ckbody, ct);
+        // (segbody: the first segment has been reversed last, whether it was run
+        // again from its checkpoint or is the only one, which has none)
+        com_tangent_kernel<<<(ctx->G.n_triangles + 255) / 256, 256, 0, s>>>(ctx->G, segbody, cpart, cticket, ct);
+        initial_spin_kernel<<<1, 32, 0, s>>>(badj, segbody, ct);
     }
     if (body) theta_reduce_kernel<<<1, 256, 0, s>>>(tslots, cap, acc);
     ADJ_CUDA(cudaMemcpyAsync(accv, acc, 3 * sizeof(double), cudaMemcpyDeviceToHost, s), "theta");

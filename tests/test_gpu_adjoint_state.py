@@ -1,0 +1,54 @@
+"""What a gradient call takes from the state before it and leaves behind: the free yaw's initial spin whatever the number
+of segments, the body after odd and even horizons, the body after a call that fails, and the memory that it asks for."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _allocator(lat):
+    """Blocks that hold NaNs (0xFF bytes) where nothing has been written; returns the sizes asked for."""
+    live, sizes = {}, []
+
+    def alloc(n, stream):
+        t = torch.full((n,), 0xFF, dtype=torch.uint8, device=lat.device)
+        torch.cuda.synchronize()
+        live[t.data_ptr()] = t
+        sizes.append(n)
+        return t.data_ptr()
+
+    lat.use_allocator(alloc, lambda p, stream: live.pop(p))
+    return sizes
+
+
+def _swimmer(free, shape=(48, 24, 24)):
+    """A turning swimmer in the centre-of-mass frame."""
+    import paper_1608_04658_gb300 as lbm
+    rest, tris = synth.swimmer_mesh(24.0, 48, 16)
+    rho, u, xi = synth.parity_fields(shape, 47)
+    lat = lbm.Lattice(shape, 0.02, storage="fp64")
+    sizes = _allocator(lat)
+    lat.set_geometry(lbm.swimmer((24.137, 12.371, 12.293), rest, tris, 24.0, 0.125, 24.0, 96.0, free=free, mass=synth.swimmer_volume(24.0),
+                                 U=(-0.01, 0.004, 0.0), psi=0.1, omega=0.003))
+    lat.init_state(rho, 0.2 * u, xi, 1e-3)
+    return lat, sizes
+
+
+@pytest.mark.parametrize("free", [4, 7])
+@pytest.mark.parametrize("horizon", [1, 2, 5, 12])
+def test_spin_gradient_does_not_depend_on_the_segments(free, horizon):
+    """K = horizon is one segment, K = 1 as many as there are steps; with the default of ceil(sqrt(horizon)) horizons 1 and
+    2 are one segment too.  Equal but for the order of the double atomics into the band slots (1e-12, as for the held
+    swimmer)."""
+    res = []
+    for K in (horizon, 1, 4, 0):
+        lat, _ = _swimmer(free)
+        res.append(lat.adjoint(horizon, (-1.0, 0.0, 0.0), want_lambda0=True, checkpoint_every=K))
+        lat.close()
+    assert np.all(np.isfinite(res[0]["dJ_dtheta"])) and np.abs(res[0]["dJ_dtheta"]).max() > 0
+    for r in res[1:]:
+        assert r["J"] == res[0]["J"]
+        assert np.allclose(r["dJ_dtheta"], res[0]["dJ_dtheta"], rtol=1e-12, atol=1e-14 * np.abs(res[0]["dJ_dtheta"]).max())
