@@ -1464,7 +1464,7 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
     BodyAdjoint hbadj{};
     DevBody hb{};
     int p = 0;
-    const int save_bcur = ctx->bcur;
+    int end_bcur = ctx->bcur;  // the body copy after the horizon (each step takes the other one)
     const int nparts = 1024;
     double Jt = 0.0;
 
@@ -1556,6 +1556,7 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
     }
     ADJ_CUDA(cudaMemcpyAsync(&hb, ctx->S.body + ctx->bcur, sizeof(DevBody), cudaMemcpyDeviceToHost, s), "body read");
     ADJ_CUDA(cudaMemcpyAsync(savebody, ctx->S.body, 2 * sizeof(DevBody), cudaMemcpyDeviceToDevice, s), "body save");
+    end_bcur = ctx->bcur;
     if (spec->lambda_T) {
         terminal_kernel<S><<<nparts, 256, 0, s>>>(L, (const S *)ctx->f[ctx->cur], (const R *)spec->lambda_T,
                                                   body ? ctx->flags : nullptr, part);
@@ -1670,7 +1671,7 @@ done:
     ctx->G.mesh_dvy = nullptr;
     // the context keeps the state after the horizon; restore its body copies
     cudaMemcpyAsync(ctx->S.body, savebody, 2 * sizeof(DevBody), cudaMemcpyDeviceToDevice, s);
-    ctx->bcur = save_bcur;
+    ctx->bcur = end_bcur;
     cudaStreamSynchronize(s);
     return st;
 }

@@ -52,3 +52,33 @@ def test_spin_gradient_does_not_depend_on_the_segments(free, horizon):
     for r in res[1:]:
         assert r["J"] == res[0]["J"]
         assert np.allclose(r["dJ_dtheta"], res[0]["dJ_dtheta"], rtol=1e-12, atol=1e-14 * np.abs(res[0]["dJ_dtheta"]).max())
+
+
+def _sphere(storage, shape=(24, 20, 22)):
+    import paper_1608_04658_gb300 as lbm
+    rho, u, xi = synth.parity_fields(shape, 4)
+    lat = lbm.Lattice(shape, 0.02, storage=storage, faces=(1, 1, 1, 1, 0, 0))
+    lat.set_geometry(lbm.sphere((11.37, 9.61, 10.83), 4.3, U=(0.02, -0.01, 0.03), free=True, g=(0, 0, -1e-4)))
+    lat.init_state(rho, 0.3 * u, xi, 1e-3)
+    return lat
+
+
+def _same_body(a, b):
+    return all(np.array_equal(np.asarray(a[k]), np.asarray(b[k])) for k in a if k != "n_band")
+
+
+@pytest.mark.parametrize("storage", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("horizon,K", [(1, 0), (2, 0), (3, 0), (3, 1), (3, 3), (4, 0), (7, 2)])
+def test_context_goes_on_as_after_the_steps(storage, horizon, K):
+    """The body, the populations and the steps that follow are those of lbm_step, bit for bit."""
+    lat, ref = _sphere(storage), _sphere(storage)
+    for l in (lat, ref):
+        l.set_launch_order("split")
+    lat.adjoint(horizon, (1.0, 0.0, 0.5), checkpoint_every=K)
+    ref.step(horizon)
+    for _ in range(3):
+        assert _same_body(lat.body(), ref.body())
+        fluid = (ref.flags & 1) == 0
+        assert torch.equal(lat.flags, ref.flags) and torch.equal(lat.f[:, fluid], ref.f[:, fluid])
+        lat.step(1)
+        ref.step(1)
