@@ -140,7 +140,9 @@ cudaError_t launch_after(bool early, void (*kernel)(K...), dim3 grid, int thread
     c.stream = s;
     c.attrs = &at;
     c.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&c, kernel, static_cast<K>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, static_cast<K>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // reported here, not by the next launch that asks for it
+    return e;
 }
 
 // Calls fn with a null pointer of the storage type (one instantiation per
