@@ -1464,7 +1464,7 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
     BodyAdjoint hbadj{};
     DevBody hb{};
     int p = 0;
-    int end_bcur = ctx->bcur;  // the body copy after the horizon (each step takes the other one)
+    int end_bcur = -1;  // the body copy after the horizon (each step takes the other one), once the copies are saved
     const int nparts = 1024;
     double Jt = 0.0;
 
@@ -1669,9 +1669,12 @@ done:
     use_slot(ctx, live);
     ctx->G.mesh_dy = nullptr;
     ctx->G.mesh_dvy = nullptr;
-    // the context keeps the state after the horizon; restore its body copies
-    cudaMemcpyAsync(ctx->S.body, savebody, 2 * sizeof(DevBody), cudaMemcpyDeviceToDevice, s);
-    ctx->bcur = end_bcur;
+    // the context keeps the state after the horizon; restore its body copies (a
+    // forward run that failed has left its own, and saved none)
+    if (end_bcur >= 0) {
+        cudaMemcpyAsync(ctx->S.body, savebody, 2 * sizeof(DevBody), cudaMemcpyDeviceToDevice, s);
+        ctx->bcur = end_bcur;
+    }
     cudaStreamSynchronize(s);
     return st;
 }

@@ -82,3 +82,18 @@ def test_context_goes_on_as_after_the_steps(storage, horizon, K):
         assert torch.equal(lat.flags, ref.flags) and torch.equal(lat.f[:, fluid], ref.f[:, fluid])
         lat.step(1)
         ref.step(1)
+
+
+def test_failed_forward_run_leaves_the_body_alone():
+    """More rows than a grid has (65,535): the forward run's first bulk launch is refused, before anything of the body has
+    been saved to be restored."""
+    import paper_1608_04658_gb300 as lbm
+    shape = (12, 65540, 12)
+    lat = lbm.Lattice(shape, 0.02, storage="fp16")
+    _allocator(lat)
+    lat.set_geometry(lbm.sphere((5.7, 30000.3, 6.1), 3.3, U=(0.02, -0.01, 0.03), free=True))
+    lat.init_state(torch.ones(shape[::-1], device=lat.device), torch.zeros((*shape[::-1], 3), device=lat.device))
+    before = lat.body()
+    with pytest.raises(lbm.LbmError):
+        lat.adjoint(3, (1.0, 0.0, 0.0))
+    assert _same_body(lat.body(), before)
