@@ -25,6 +25,7 @@ __device__ __forceinline__ Pair32 operator+(Pair32 a, Pair32 b)
     return {s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
 }
 __device__ __forceinline__ Pair32 operator-(Pair32 a, Pair32 b) { return a + Pair32{-b.hi, -b.lo}; }
+// (without lo^2: added here, it would be rounded away more often than not)
 __device__ __forceinline__ Pair32 square(Pair32 a)
 {
     const float p = __fmul_rn(a.hi, a.hi);

@@ -99,6 +99,9 @@ struct NodeTotals<float> {
     static constexpr int FLUSH = 16;
     double acc[5] = {0, 0, 0, 0, 0};
     Pair32 part[5] = {};
+    // what the squares of the pairs leave out, lo^2: of one sign, so that it does
+    // not average out over the nodes (3e-15 of the kinetic energy in FP32)
+    float squares = 0.f;
     int held = 0;
     long long count = 0;
     __device__ __forceinline__ void flush()
@@ -108,6 +111,8 @@ struct NodeTotals<float> {
             acc[k] += value(part[k]);
             part[k] = Pair32{0.f, 0.f};
         }
+        acc[4] += (double)squares;
+        squares = 0.f;
         held = 0;
     }
     __device__ __forceinline__ void add(const float (&g)[Q], double rho0)
@@ -117,10 +122,13 @@ struct NodeTotals<float> {
         const float r0 = (float)rho0;
         const Pair32 rho = Pair32{r0, (float)(rho0 - (double)r0)} + m[0];
         const Pair32 q = (square(m[1]) + square(m[2])) + square(m[3]);
-        // quotient q / rho: the FP32 one and its remainder's
+        // quotient q / rho: the FP32 one and its remainder's, the second with what
+        // the reciprocal leaves of it (inv (1 + e1)): the square of the
+        // reciprocal's error has one sign, 1e-15 of the sum
         const float inv = rcp_fast(rho.hi), k1 = __fmul_rn(q.hi, inv);
         const float rem = __fadd_rn(__fmaf_rn(-k1, rho.hi, q.hi), __fmaf_rn(-k1, rho.lo, q.lo));
-        const Pair32 ke = two_sum(k1, __fmul_rn(rem, inv));
+        const float e1 = __fmaf_rn(-rho.lo, inv, __fmaf_rn(-rho.hi, inv, 1.f)), k2 = __fmul_rn(rem, inv);
+        const Pair32 ke = two_sum(k1, __fmaf_rn(k2, e1, k2));
         // the range in which the pairs' products neither overflow nor lose
         // their remainders to underflow
         if (rho.hi > 1e-6f && rho.hi < 1e6f && fabsf(m[0].hi) < 1e6f && q.hi < 1e12f &&
@@ -129,6 +137,7 @@ struct NodeTotals<float> {
 #pragma unroll
             for (int k = 0; k < 4; ++k) part[k] = part[k] + m[k];
             part[4] = part[4] + ke;
+            squares = __fmaf_rn(__fmaf_rn(m[1].lo, m[1].lo, __fmaf_rn(m[2].lo, m[2].lo, __fmul_rn(m[3].lo, m[3].lo))), inv, squares);
             if (++held == FLUSH) flush();
         } else {
             double t[5];
