@@ -101,9 +101,10 @@ template <> struct ForceSlot<double> {
     int k;
 };
 template <> struct ForceSlot<float> {
-    float hi[3], lo[3], h[3];
+    float hi[3], lo[3], h[3], hl[3];
     int k;
 };
+static_assert(sizeof(ForceSlot<float>) <= FORCE_SLOT * sizeof(double) && sizeof(ForceSlot<double>) <= FORCE_SLOT * sizeof(double), "force slot");
 __host__ __device__ constexpr int weight216(int i) { return nonzero_of(i) == 0 ? 64 : nonzero_of(i) == 1 ? 16 : nonzero_of(i) == 2 ? 4 : 1; }
 // |k| <= 36 each
 __host__ __device__ constexpr int pack_k(int a, int b, int c) { return (a + 128) | (b + 128) << 8 | (c + 128) << 16; }

@@ -28,8 +28,7 @@
 //   Refill: mean density of the neighbours fluid at t (rho0 if none), the body
 //   velocity (the swimmer's material velocity at the node's arc position),
 //   gradient with the wall velocity at the centre.
-#include "lanes.cuh"
-#include "pair32.cuh"
+#include "force.cuh"
 
 namespace lbm {
 
@@ -40,90 +39,6 @@ namespace lbm {
 #ifndef LBM_LIST_MIN_BLOCKS
 #define LBM_LIST_MIN_BLOCKS 7
 #endif
-
-// A boundary node's sums over its links into its slot (see ForceSlot).  FP32
-// and 16-bit storage: sums of -c (f_out + f_in) + u_w (f_in - f_out) without
-// W rho0 as pairs hi + lo of FP32 numbers, error-free but for 2^-48 of values a
-// hundredth of f; W rho0 as the integer sum of 216 W c.  FP64 arithmetic here
-// runs with a fifth of the lanes at work (the missing links of one node) on a
-// pipe of two lanes a clock and SM: it took the larger part of this kernel's
-// time (airfoil 225 us with it).  The force kernel does it for 32 nodes a warp.
-template <typename R>
-__device__ __forceinline__ void node_force(double *slot, int lane, bool link, int cx, int cy, int cz,
-                                           int i, R fbb, R gi, R q, const R uw[3], const float ul[3]);
-template <>
-__device__ __forceinline__ void node_force<double>(double *slot, int lane, bool link, int cx, int cy,
-                                                   int cz, int i, double fbb, double gi, double q, const double uw[3],
-                                                   const float ul[3])
-{
-    // force without W rho0, and -sum q (f_in - f_out) (c x u_w)
-    double v[6] = {0, 0, 0, 0, 0, 0};
-    if (link) {
-        const double sum = fbb + gi, dif = gi - fbb, h = -q * dif;
-        const int c[3] = {cx, cy, cz};
-        for (int a = 0; a < 3; ++a) {
-            v[a] = fma(uw[a], dif, c[a] == 0 ? 0.0 : (c[a] > 0 ? -sum : sum));
-            const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
-            v[3 + a] = h * (c[b1] * uw[b2] - c[b2] * uw[b1]);
-        }
-    }
-    const double s = wsum_scatter6(v, lane);
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-        if (lane == wsum_owner6(k)) reinterpret_cast<ForceSlot<double> *>(slot)->v[k] = s;
-    const int w = link ? weight216(i) : 0;
-    const int k0 = __reduce_add_sync(FULL, w * cx), k1 = __reduce_add_sync(FULL, w * cy),
-              k2 = __reduce_add_sync(FULL, w * cz);
-    if (lane == 0) reinterpret_cast<ForceSlot<double> *>(slot)->k = pack_k(k0, k1, k2);
-}
-template <>
-__device__ __forceinline__ void node_force<float>(double *slot, int lane, bool link, int cx, int cy,
-                                                  int cz, int i, float fbb, float gi, float q, const float uw[3],
-                                                  const float ul[3])
-{
-    Pair32 F[3] = {};
-    float H[3] = {0.f, 0.f, 0.f};
-    if (link) {
-        const Pair32 sum = two_sum(fbb, gi), dif = two_sum(gi, -fbb);
-        const int c[3] = {cx, cy, cz};
-        for (int a = 0; a < 3; ++a) {
-            const Pair32 p = Pair32{uw[a], ul[a]} * dif;
-            F[a] = c[a] == 0 ? p : (c[a] > 0 ? p - sum : p + sum);
-        }
-        const float h = -q * dif.hi;
-        for (int a = 0; a < 3; ++a) {
-            const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
-            H[a] = h * (c[b1] * uw[b2] - c[b2] * uw[b1]);
-        }
-    }
-    // sums as in wsum_scatter6: component 2 to the upper half of the warp, 1 to
-    // the upper quarter of the lower half
-    const auto exchange = [&](Pair32 a, Pair32 b, int o) {
-        const bool up = lane & o;
-        const Pair32 keep = up ? b : a, send = up ? a : b;
-        return keep + Pair32{__shfl_xor_sync(FULL, send.hi, o), __shfl_xor_sync(FULL, send.lo, o)};
-    };
-    const Pair32 none = {0.f, 0.f}, F02 = exchange(F[0], F[2], 16), F1 = exchange(F[1], none, 16);
-    const float H02 = wexchange(H[0], H[2], lane, 16), H1 = wexchange(H[1], 0.f, lane, 16);
-    Pair32 Fs = exchange(F02, F1, 8);
-    float Hs = wexchange(H02, H1, lane, 8);
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        Fs = Fs + Pair32{__shfl_xor_sync(FULL, Fs.hi, o), __shfl_xor_sync(FULL, Fs.lo, o)};
-        Hs += __shfl_xor_sync(FULL, Hs, o);
-    }
-    const int w = link ? weight216(i) : 0;
-    const int k0 = __reduce_add_sync(FULL, w * cx), k1 = __reduce_add_sync(FULL, w * cy),
-              k2 = __reduce_add_sync(FULL, w * cz);
-    ForceSlot<float> *p = reinterpret_cast<ForceSlot<float> *>(slot);
-    if ((lane & 7) == 0 && lane < 24) {
-        const int a = lane >> 3;  // lane 0, 8, 16: components 0, 1, 2
-        p->hi[a] = Fs.hi;
-        p->lo[a] = Fs.lo;
-        p->h[a] = Hs;
-    }
-    if (lane == 0) p->k = pack_k(k0, k1, k2);
-}
 
 template <typename S>
 __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_kernel(
@@ -194,6 +109,9 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
             link_data<R>(L, G, b, s_wall.air, x, y, z, i, q, uw, ul);
         }
         const R qq = (R)q;
+        // (the airfoil's and the swimmer's links are found in the precision of R)
+        float ql = 0.f;
+        if (sizeof(R) == 4 && (G.kind == LBM_BODY_SPHERE || G.kind == LBM_BODY_PLANES)) ql = (float)(q - (double)qq);
         const R gstat = miss ? fbb : Fi;
         const R dyn = miss ? R(6) * weight<R>(i) * rho0 * (R(cx) * uw[0] + R(cy) * uw[1] + R(cz) * uw[2]) : R(0);
         R ut[3] = {0, 0, 0};
@@ -223,7 +141,7 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
         // into its band slot, which the force kernel turns into force and torque
         // a slab's links count where it owns the fluid node
         const bool own = z >= G.own_lo && z < G.own_hi;
-        node_force<R>(bforce + (size_t)bpos[slot] * FORCE_SLOT, lane, own && miss, cx, cy, cz, i, fbb, gi, qq, uw, ul);
+        node_force<R>(bforce + (size_t)bpos[slot] * FORCE_SLOT, lane, own && miss, cx, cy, cz, i, fbb, gi, qq, ql, uw, ul);
 
         bool ok;
         const R out = kbc_collide_lanes<R>(gi, i, (R)L.beta, (R)L.inv_beta, rho0, L.gamma_mode, ok);

@@ -16,7 +16,7 @@
 //             depend on list order or block timing.
 #include <algorithm>
 
-#include "lanes.cuh"
+#include "force.cuh"
 
 namespace lbm {
 
@@ -396,24 +396,12 @@ __global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Lattice L, c
         used = true;
         const int k = spos[threadIdx.x];
         band_node(L, G, lo, cnt, k, x, y, z);
-        const ForceSlot<R> *p = reinterpret_cast<const ForceSlot<R> *>(bforce + (size_t)k * FORCE_SLOT);
-        double F[3], h[3];
-        const int kk = p->k;
-        for (int a = 0; a < 3; ++a) {
-            if constexpr (sizeof(R) == 8) {
-                F[a] = p->v[a];
-                h[a] = p->v[3 + a];
-            } else {
-                F[a] = (double)p->hi[a] + (double)p->lo[a];
-                h[a] = (double)p->h[a];
-            }
-            F[a] -= (L.rho0 / 108.0) * unpack_k(kk, a);
-        }
         const double o[3] = {body_offset(L, G, cur, 0, x), body_offset(L, G, cur, 1, y), body_offset(L, G, cur, 2, z)};
+        double F[3], M[3];
+        slot_force<R>(bforce + (size_t)k * FORCE_SLOT, L.rho0, o, F, M);
         for (int a = 0; a < 3; ++a) {
-            const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
             acc[a] += F[a];
-            acc[3 + a] += o[b1] * F[b2] - o[b2] * F[b1] + h[a];
+            acc[3 + a] += M[a];
         }
     }
     __shared__ double sm[FORCE_THREADS / 32][6];
