@@ -141,7 +141,14 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) boundary_ker
         // into its band slot, which the force kernel turns into force and torque
         // a slab's links count where it owns the fluid node
         const bool own = z >= G.own_lo && z < G.own_hi;
-        node_force<R>(bforce + (size_t)bpos[slot] * FORCE_SLOT, lane, own && miss, cx, cy, cz, i, fbb, gi, qq, ql, uw, ul);
+        double *fslot = bforce + (size_t)bpos[slot] * FORCE_SLOT;
+        if (__any_sync(FULL, miss && force_overflows<R>(fbb, gi, uw))) {
+            const double o[3] = {body_offset(L, G, b, 0, x), body_offset(L, G, b, 1, y), body_offset(L, G, b, 2, z)};
+            const double ud[3] = {(double)uw[0] + (double)ul[0], (double)uw[1] + (double)ul[1], (double)uw[2] + (double)ul[2]};
+            force_plain(fslot, lane, own && miss, i, (double)fbb, (double)gi, q, ud, o, L.rho0);
+        } else {
+            node_force<R>(fslot, lane, own && miss, cx, cy, cz, i, fbb, gi, qq, ql, uw, ul);
+        }
 
         bool ok;
         const R out = kbc_collide_lanes<R>(gi, i, (R)L.beta, (R)L.inv_beta, rho0, L.gamma_mode, ok);

@@ -3,6 +3,8 @@
 // reads from them.
 #pragma once
 
+#include <cstddef>
+
 #include "lanes.cuh"
 #include "pair32.cuh"
 
@@ -95,13 +97,61 @@ __device__ __forceinline__ void node_force<float>(double *slot, int lane, bool l
     if (lane == 0) p->k = pack_k(k0, k1, k2);
 }
 
+// What a node leaves whose sums overflow, or whose state is no longer finite:
+// force and torque themselves (o: the node's offset from the reference point),
+// in FP64 from the full populations, link by link, so that an infinite
+// population gives the infinities and NaNs of the momentum exchange and not
+// those of how it is evaluated.  Out of line, no node of a stable run takes it.
+constexpr int SLOT_PLAIN = 1 << 24;
+__device__ __noinline__ static void force_plain(double *slot, int lane, bool link, int i, double fbb, double gi, double q,
+                                                const double uw[3], const double o[3], double rho0)
+{
+    double v[6] = {0, 0, 0, 0, 0, 0};
+    if (link) {
+        const double W = weight<double>(i) * rho0, fout = fbb + W, fin = gi + W;
+        const double c[3] = {(double)cx_of(i), (double)cy_of(i), (double)cz_of(i)};
+        double r[3];
+        for (int a = 0; a < 3; ++a) {
+            v[a] = (-c[a] - uw[a]) * fout - (c[a] - uw[a]) * fin;
+            r[a] = o[a] - q * c[a];
+        }
+        v[3] = r[1] * v[2] - r[2] * v[1];
+        v[4] = r[2] * v[0] - r[0] * v[2];
+        v[5] = r[0] * v[1] - r[1] * v[0];
+    }
+    const double s = wsum_scatter6(v, lane);
+    ForceSlot<double> *p = reinterpret_cast<ForceSlot<double> *>(slot);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (lane == wsum_owner6(k)) p->v[k] = s;
+    if (lane == 0) p->k = SLOT_PLAIN;
+}
+
+// whether a link's values are outside the range in which the sums of the other
+// form can neither overflow nor lose their low parts
+template <typename R>
+__device__ __forceinline__ bool force_overflows(R fbb, R gi, const R uw[3])
+{
+    const R big = sizeof(R) == 4 ? R(1e30) : R(1e290);
+    return !(fabs(fbb) + fabs(gi) < big && fabs(uw[0]) + fabs(uw[1]) + fabs(uw[2]) < R(1e6));
+}
+
 // The node's force F and torque M about the reference point from its slot; o:
 // its offset from there (see ForceSlot).
 template <typename R>
 __device__ __forceinline__ void slot_force(const double *slot, double rho0, const double o[3], double F[3], double M[3])
 {
+    static_assert(offsetof(ForceSlot<float>, k) == offsetof(ForceSlot<double>, k), "a plain slot is told by its k");
     const ForceSlot<R> *p = reinterpret_cast<const ForceSlot<R> *>(slot);
     const int k = p->k;
+    if (k & SLOT_PLAIN) {
+        const ForceSlot<double> *w = reinterpret_cast<const ForceSlot<double> *>(slot);
+        for (int a = 0; a < 3; ++a) {
+            F[a] = w->v[a];
+            M[a] = w->v[3 + a];
+        }
+        return;
+    }
     double h[3];
     for (int a = 0; a < 3; ++a) {
         if constexpr (sizeof(R) == 8) {
