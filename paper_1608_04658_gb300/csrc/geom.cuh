@@ -279,20 +279,27 @@ struct TriF {
             r[a] = -pa;
         }
     }
-    // crossing of the link from p along -c at p - sv c, with its barycentric
-    // coordinates
-    __device__ __forceinline__ bool hit(const int c[3], float &sv, float &uf, float &vf) const
+    // where the line of the link from p along -c meets the triangle's plane: p -
+    // s c, with its barycentric coordinates (false: parallel)
+    __device__ __forceinline__ bool meet(const int c[3], float &s, float &u, float &v) const
     {
-        constexpr float EPS = 1e-6f;
         const float dc[3] = {(float)c[0], (float)c[1], (float)c[2]};
         const float D = det3f(e1, e2, dc);
         if (D == 0.0f) return false;
         const float iD = 1.0f / D;
-        uf = det3f(r, e2, dc) * iD;
-        vf = det3f(e1, r, dc) * iD;
-        const float sf = det3f(e1, e2, r) * iD;
-        if (uf < -EPS || vf < -EPS || uf + vf > 1.0f + EPS || sf < -EPS || sf > 1.0f + EPS) return false;
-        sv = fminf(fmaxf(sf, 0.0f), 1.0f);
+        u = det3f(r, e2, dc) * iD;
+        v = det3f(e1, r, dc) * iD;
+        s = det3f(e1, e2, r) * iD;
+        return true;
+    }
+    // whether the link crosses the triangle, and its fraction there
+    __device__ __forceinline__ bool hit(const int c[3], float &sv) const
+    {
+        constexpr float EPS = 1e-6f;
+        float s, u, v;
+        if (!meet(c, s, u, v)) return false;
+        if (u < -EPS || v < -EPS || u + v > 1.0f + EPS || s < -EPS || s > 1.0f + EPS) return false;
+        sv = fminf(fmaxf(s, 0.0f), 1.0f);
         return true;
     }
 };
@@ -349,8 +356,8 @@ __device__ __forceinline__ void mesh_first_crossings(const GeomParams &G, const 
     const auto test = [&](unsigned pair) {
         const int i = pair & 31, k = pair >> 5;
         const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
-        float sv, u, v;
-        if (TriF(G, k, p).hit(c, sv, u, v))
+        float sv;
+        if (TriF(G, k, p).hit(c, sv))
             atomicMin(S.key + i, (unsigned long long)__float_as_uint(sv + 0.0f) << 32 | (unsigned)k);
     };
     int queued = 0;
@@ -412,12 +419,15 @@ __device__ void mesh_links_warp(const GeomParams &G, const DevBody *b, int x, in
             const unsigned long long kk = S.key[lane];
             if (kk != ~0ull) {
                 const int c[3] = {cx_of(lane), cy_of(lane), cz_of(lane)};
-                float sv = 0.f, u = 0.f, v = 0.f;
+                // (the fraction is the one that was accepted; the coordinates are
+                // formed again without the test, which a different rounding here
+                // could fail at its edge)
+                float s = 0.f, u = 0.f, v = 0.f;
                 hitout.tri = (int)(unsigned)kk;
-                TriF(G, hitout.tri, p).hit(c, sv, u, v);
+                TriF(G, hitout.tri, p).meet(c, s, u, v);
                 hitout.u = u;
                 hitout.v = v;
-                q = sv;
+                q = __uint_as_float((unsigned)(kk >> 32));
             }
         }
         __syncwarp();
