@@ -126,13 +126,12 @@ __device__ __forceinline__ void kbc_vjp_v(typename O::V (&g)[Q], typename O::V (
     }
     // the stabilizer and the adjoints of a and b; where f is an equilibrium to
     // rounding the stabilizer is 2 and constant
-    const V k0 = O::rcp(O::mul(O::mul(rho, O::c(8.0 / 27.0)), O::mul(X.phi(0), O::mul(Y.phi(0), Z.phi(0)))));
     R abv[NL], bbv[NL], chv[NL];
     const R kk = O1<R>::sub(R(2), inv_beta);
 #pragma unroll
     for (int k = 0; k < NL; ++k) {
         const R shk = O::lane(sh, k), hhk = O::lane(hh, k);
-        const bool analytic = gamma_mode == LBM_GAMMA_ANALYTIC && O1<R>::mul(hhk, O::lane(k0, k)) > gamma_floor<R>();
+        const bool analytic = gamma_mode == LBM_GAMMA_ANALYTIC && has_stabilizer(hhk, O::lane(rho, k));
         const R ihh = analytic ? rcp_fast(hhk) : R(0);
         const R ratio = O1<R>::mul(shk, ihh);
         const R gam = analytic ? O1<R>::sub(inv_beta, O1<R>::mul(kk, ratio)) : R(2);

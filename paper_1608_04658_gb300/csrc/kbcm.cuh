@@ -62,6 +62,19 @@ struct Shear {
     __device__ __forceinline__ V at(int i) const { return shear_v<V>(i, sx, sy, sz, qxy, qxz, qyz); }
 };
 
+// Whether a node's stabilizer is defined (gamma_floor, where f is an equilibrium
+// to rounding it is 2), for a product hh = <dh|dh> taken with 1/f^eq relative to
+// the rest direction's, 27/(8 rho): hh goes with rho^2, the floor is one of
+// <dh|dh> itself, which goes with rho.  The second bound keeps 1/hh finite.
+__device__ __forceinline__ bool has_stabilizer(float hh, float rho)
+{
+    return hh > gamma_floor<float>() * (float)(8.0 / 27.0) * rho && hh > 1.2e-38f;
+}
+__device__ __forceinline__ bool has_stabilizer(double hh, double rho)
+{
+    return hh > gamma_floor<double>() * (8.0 / 27.0) * rho && hh > 2.3e-308;
+}
+
 // Root of Eq. (gamma_min) per lane from the analytic value gam (see
 // exact_gamma): with x_i = f'_i(gam)/f^eq_i - 1 and t_i = b dh_i/f'_i(gam),
 //   r(gam + s) = sum dh_i log(1 + x_i) - s sum dh_i t_i - s^2/2 sum dh_i t_i^2 - ...,
@@ -130,7 +143,7 @@ __device__ __forceinline__ int exact_stabilizer(const typename O::V (&d)[Q], con
     int again = 0;
 #pragma unroll
     for (int k = 0; k < NL; ++k) {
-        if (!(O::lane(hh, k) > gamma_floor<R>())) continue;
+        if (!has_stabilizer(O::lane(hh, k), O::lane(rho, k))) continue;
         const R f0 = O::lane(r0, k), f1 = O::lane(r1, k), f2 = O::lane(r2, k), i1 = rcp_fast(f1);
         const R s1 = f0 * i1;
         const R s = s1 - R(0.5) * f2 * s1 * s1 * rcp_fast(f1 + f2 * s1);
@@ -290,7 +303,7 @@ __device__ __forceinline__ int kbc_collide_m(typename O::V (&g)[Q], typename O::
     for (int k = 0; k < NL; ++k) {
         const R shk = O::lane(sh, k), hhk = O::lane(hh, k);
         gam[k] = R(2);
-        if (gamma_mode != LBM_GAMMA_LBGK && hhk > gamma_floor<R>())
+        if (gamma_mode != LBM_GAMMA_LBGK && has_stabilizer(hhk, O::lane(rho, k)))
             gam[k] = O1<R>::sub(inv_beta, O1<R>::mul(O1<R>::mul(O1<R>::sub(R(2), inv_beta), shk), rcp_fast(hhk)));
     }
     if constexpr (EXACT) {
