@@ -318,8 +318,9 @@ LBM_API lbm_status lbm_reset_average(lbm_ctx *ctx);
 LBM_API lbm_status lbm_save(lbm_ctx *ctx, const char *path);
 LBM_API lbm_status lbm_load(lbm_ctx *ctx, const char *path);
 
-/* Mass, momentum (3) and kinetic energy summed over fluid nodes in double,
- * written to host out[5].  Synchronises. */
+/* Mass, momentum (3) and kinetic energy summed over fluid nodes in double (FP32
+ * and 16-bit storage: a node's own sums, and those of up to 16 nodes, as pairs
+ * of floats of some 48 bits), written to host out[5].  Synchronises. */
 LBM_API lbm_status lbm_totals(lbm_ctx *ctx, double out[5]);
 
 /* Launch order of the steps of a body whose band is known before its
@@ -390,9 +391,13 @@ LBM_API lbm_status lbm_profile_end(lbm_ctx *ctx, double *total_ms, int64_t *laun
  *
  * Memory: the forward states are kept by checkpoint-and-recompute: every
  * checkpoint_every steps (0: ceil(sqrt(horizon))) a state is kept, and each
- * segment but the last is recomputed once during the reverse sweep; the call
- * allocates at most (ceil(horizon/K) + K + 1) state buffers of 27 N elements and
- * frees them before returning (LBM_ERR_OOM if they do not fit).
+ * segment but the last is recomputed once during the reverse sweep.  With K
+ * steps a segment (at most horizon) the call allocates ceil(horizon/K) + K - 1
+ * buffers of 27 N elements of the storage type, two of 27 N elements of the
+ * adjoint's (double for FP64 storage, float for the others: for 16-bit storage
+ * these count as four), (ceil(horizon/K) + K + 4) N bytes of marks, and with a
+ * body K copies of its lists and mesh arrays and 72 doubles per node of its
+ * band; it frees them before returning (LBM_ERR_OOM if they do not fit).
  *
  * On return the context has advanced by horizon steps, exactly as
  * lbm_step(horizon) would have (the forces of those steps are in the body

@@ -97,3 +97,19 @@ def test_failed_forward_run_leaves_the_body_alone():
     with pytest.raises(lbm.LbmError):
         lat.adjoint(3, (1.0, 0.0, 0.0))
     assert _same_body(lat.body(), before)
+
+
+@pytest.mark.parametrize("storage,es,rs", [("fp64", 8, 8), ("fp32", 4, 4), ("fp16", 2, 4)])
+@pytest.mark.parametrize("horizon,K", [(1, 1), (7, 3), (9, 9)])
+def test_memory_asked_for(storage, es, rs, horizon, K):
+    """What include/lbm.h says of a box without a body: ceil(horizon/K) + K - 1 states in the storage type, two in the
+    adjoint's, (ceil(horizon/K) + K + 4) N bytes of marks (and a few kilobytes)."""
+    import paper_1608_04658_gb300 as lbm
+    shape = (40, 32, 24)
+    N, nseg = 40 * 32 * 24, -(-horizon // K)
+    lat = lbm.Lattice(shape, 0.02, storage=storage)
+    sizes = _allocator(lat)
+    lat.init_state(*synth.uniform_fields(shape))
+    lat.adjoint(horizon, lambda_T=torch.ones((27,) + shape[::-1], device=lat.device), checkpoint_every=K)
+    bound = (nseg + K - 1) * 27 * N * es + 2 * 27 * N * rs + (nseg + K + 4) * N + 65536
+    assert 0.9 * bound < sum(sizes) <= bound
