@@ -50,7 +50,7 @@ BYTES_PER_NODE = {"fp64": 432, "fp32": 216, "fp16": 108, "bf16": 108}
 DTYPE = {"fp64": "f64", "fp32": "f32", "fp16": "f32", "bf16": "f32"}
 FALLBACK_HBM_GBS = 6800.0
 PROFILES = os.path.join(ROOT, "profiles")
-KERNEL_SOURCES = ["bulk.cu", "bulk.cuh", "pull.cuh", "kbc.cuh", "kbcv.cuh", "kbcm.cuh", "lbm_internal.cuh"]
+KERNEL_SOURCES = ["bulk.cu", "bulk_fp32.cu", "bulk_fp16.cu", "bulk_bf16.cu", "bulk.cuh", "pull.cuh", "kbc.cuh", "kbcv.cuh", "kbcm.cuh", "lbm_internal.cuh"]
 
 
 def parse_args(argv=None):

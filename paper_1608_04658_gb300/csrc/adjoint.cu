@@ -1022,8 +1022,8 @@ __global__ void __launch_bounds__(BWARPS * 32) adjoint_refill_kernel(
 
 // theta-tangents of every mesh vertex at the pose of body state b[j]: dy/dtheta
 // (position) and the central difference of it (velocity), 3 + 3 per vertex,
-// into dy[j] / dvy[j], for the steps j = blockIdx.y of a recomputed segment
-// at once.  One warp per block: the FP64 arithmetic spread over as many SMs
+// into dy[j] / dvy[j], for the steps j = blockIdx.y of a segment at
+// once.  One warp per block: the FP64 arithmetic spread over as many SMs
 // as there are warps, not over the few schedulers of a handful of large
 // blocks.
 constexpr int TANGENT_THREADS = 32;
@@ -1372,9 +1372,9 @@ cudaError_t reverse_step(lbm_ctx *ctx, const S *st, const NextAdj<typename Codec
 
 // The arrays a step's geometry writes and the later kernels of that step (and
 // of its reverse) read: the boundary and uncovered lists and, for the mesh,
-// the pose and the column and cell lists.  The recompute pass gives every
-// step of a segment a slot of its own, so the reversed step finds its
-// geometry there instead of running it again.
+// the pose and the column and cell lists.  Every step of a segment has a slot
+// of its own, filled when the segment is run again (the last one: by the forward
+// run), so the reversed step finds its geometry there instead of running it again.
 struct GeoSlot {
     int *blist = nullptr, *bpos = nullptr, *ulist = nullptr, *upos = nullptr;
     double *mesh_pos = nullptr, *mesh_vel = nullptr, *col_x = nullptr;
@@ -1574,7 +1574,7 @@ lbm_status adjoint_run(lbm_ctx *ctx, const lbm_adjoint *spec, double *J, double 
     *J = Jt;
     for (int a = 0; a < 3; ++a) *J += spec->w_force[a] * (F1[a] - F0[a]) / T;
 
-    // ---- reverse sweep, one recomputed segment at a time
+    // ---- reverse sweep, one segment at a time, each but the last run again first
     ADJ_CUDA(cudaMemsetAsync(acc, 0, 3 * sizeof(double), s), "clear");
     ADJ_CUDA(cudaMemsetAsync(tslots, 0, (size_t)cap * 6 * sizeof(double), s), "clear");
     ADJ_CUDA(cudaMemcpyAsync(badj, &badj0, sizeof(BodyAdjoint), cudaMemcpyHostToDevice, s), "body adjoint");

@@ -219,9 +219,9 @@ __global__ void __launch_bounds__(BWARPS * 32, LBM_LIST_MIN_BLOCKS) refill_kerne
 #ifndef LBM_LIST_BLOCKS
 #define LBM_LIST_BLOCKS 304
 #endif
-// The links of the swimmer (a triangle search) and of the airfoil (a bisection)
-// make their boundary kernel the long part of the body's launch chain:
-// LBM_LINK_LIST_BLOCKS gives it more blocks (608 took the 256x128x128
+// The links of the swimmer (a triangle search) and of the airfoil (a root on
+// the outline) make their boundary kernel the long part of the body's launch
+// chain: LBM_LINK_LIST_BLOCKS gives it more blocks (608 took the 256x128x128
 // swimmer's step from 0.359 to 0.256 ms and the two-level airfoil's coarse
 // step from 1.13 to 1.05 ms; 1064 measured 1.07).
 #ifndef LBM_LINK_LIST_BLOCKS

@@ -1,14 +1,15 @@
 // Bulk fused pull-stream + KBC collide (arXiv 1608.04658, Sec. 2, Eq. kineticEq
 // with Eq. kbc_relax).
 //
-// One thread per node, threads along x (the fastest axis of every population
-// plane) so each of the 27 plane loads and stores of a warp is one contiguous
-// run; the +-1 x-shift of a pull touches one extra 32-byte sector per warp,
-// which the neighbouring warp reads anyway, so DRAM traffic stays at one read
-// and one write per population.  Nodes marked SOLID or BOUNDARY are left to
-// the boundary kernel.  With a body, one launch takes the nodes outside the
-// body's sweep box (no flag read) while the body's geometry runs beside it,
-// and a second the nodes of the box once their marks are known.
+// Two nodes per thread (bulk_pair_kernel) or one (bulk_kernel), threads along x
+// (the fastest axis of every population plane) so each of the 27 plane loads and
+// stores of a warp is one contiguous run; the +-1 x-shift of a pull touches one
+// extra 32-byte sector per warp, which the neighbouring warp reads anyway, so
+// DRAM traffic stays at one read and one write per population.  Nodes marked
+// SOLID or BOUNDARY are left to the boundary kernel.  With a body, one launch
+// takes the nodes outside the body's sweep box (no flag read) while the body's
+// geometry runs beside it, and a second the nodes of the box once their marks
+// are known.
 #pragma once
 
 #include <algorithm>
@@ -251,13 +252,17 @@ cudaError_t launch_bulk_form(const Lattice &L, const S *fa, S *fb, const uint8_t
     return launch_after(early, bulk_kernel<S, FORM>, grid, bx, s, L, fa, fb, flags, status, sweep, mode, capx, capy, z_lo);
 }
 
-// FP32 and 16-bit boxes with a body and fewer nodes than this keep
-// kbc_collide_v: their step is bound by the body's chain (and FP32's bulk launch
-// by memory), both forms take the same time (128x128x256 sphere), and what a
-// different operation order moves there shows in sums of both signs, such as
-// the mean thrust of an adjoint's objective.  Larger ones and those without a
-// body, where the bulk launch is the step, take kbc_collide_m (768x256x256
-// FP16 1219 -> 1062 us, 1024x512x64 with faces 874 -> 767).  A slab goes by the
+// In FP32 and 16 bits a launch over every node without marks takes
+// kbc_collide_m, and so does every launch on a box of this many nodes or more
+// (768x256x256 FP16 1219 -> 1062 us, 1024x512x64 with faces 874 -> 767).  A
+// launch beside a body's chain or with marks on a smaller box (a refinement's
+// levels too, with or without a body) keeps kbc_collide_v.  Below the line it is
+// one of bits and not of time: a step in us by the one and the other form is, in
+// FP32 and FP16, 156 and 154, 132 and 121 (128x128x256 sphere), 168 and 173, 142
+// and 132 (512x256x32 airfoil), 208 and 203, 184 and 174 (256x128x128 swimmer),
+// 379 and 366, 340 and 331 (256x128x32 airfoil on two levels); the other order
+// of operations moves the rounding of a store, which shows in sums of both
+// signs, such as the mean thrust of an adjoint's objective.  A slab goes by the
 // whole box, whose bits its own layers have to give.
 constexpr long long MOMENT_FORM_NODES = 1LL << 23;
 

@@ -1,6 +1,6 @@
 // KBC collision of one node (F1, D1) or two nodes at once (F2, packed FP32x2)
-// from its moments: the form that FP64 storage, boxes without a body, large
-// ones and the exact stabilizer take (see launch_bulk_t).  Same mathematics as kbc_collide
+// from its moments: the form that FP64 storage, the exact stabilizer, launches
+// without marks and large boxes take (see launch_bulk_t).  Same mathematics as kbc_collide
 // (arXiv 1608.04658, Sec. 2, Eqs. kineticEq, kbc_relax, feq_min, gamma_min and
 // the analytic stabilizer); the one-node and the two-node FP32 forms give the
 // same bits for a node.
