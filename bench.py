@@ -592,7 +592,7 @@ def adjoint_bench(args, world, device):
             "fwd_ms_per_step": round(fwd_ms / H, 5), "adjoint_ms_per_step": round(adj_ms / H, 5),
             "adjoint_over_forward": round(adj_ms / fwd_ms, 3),
             "J": out["J"], "dJ_dtheta": [float(v) for v in out["dJ_dtheta"]],
-            "checkpoint_bytes": int((math.ceil(H / K) + K + 3) * 27 * nx * ny * nz * 4)}
+            "checkpoint_bytes": int((math.ceil(H / K) + K + 1) * 27 * nx * ny * nz * 4)}
 
 
 def accuracy_bench(args, device):
