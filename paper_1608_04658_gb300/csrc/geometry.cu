@@ -763,8 +763,14 @@ cudaError_t launch_forces(int storage, const Lattice &L, const GeomParams &G, Sc
     // and a round trip to memory (airfoil, 240,000 positions: 128 blocks 28 us)
     const long long cap = (long long)G.cap[0] * G.cap[1] * G.cap[2];
     const int nb = (int)std::min<long long>(S.n_partials, (cap + 2 * FORCE_THREADS - 1) / (2 * FORCE_THREADS));
+    // Early where no SM holds more than one of its blocks (152 SMs): they take their
+    // places while the boundary nodes run, away from the bulk launch beside those.
+    // Walls, whose band is the box, 96x64x48 and 40x128x40 in FP64: 10 steps 14.0
+    // and 7.0 ms with 576 and 400 blocks waiting, 12.3 and 5.4 so (FP32 64x64x32
+    // 1.02 and 1.03)
+    const bool early = L.short_bulk && nb <= 152;
     *nlaunch += 1;
-    return launch_after(L.short_bulk, kernel, nb, FORCE_THREADS, s, L, G, S.body + cur, flags, S.bforce, S.partials, S.ticket);
+    return launch_after(early, kernel, nb, FORCE_THREADS, s, L, G, S.body + cur, flags, S.bforce, S.partials, S.ticket);
 }
 
 cudaError_t launch_sweep_init(const Lattice &L, const GeomParams &G, Scratch &S, int cur, cudaStream_t s)
