@@ -148,7 +148,9 @@ __device__ __forceinline__ void pair_update(const Lattice &L, const S *fa, S *fb
     }
     const int n0 = x0 + L.nx * (y + L.ny * z);
     if (flags != nullptr) {
-        const unsigned fw = ODD ? flags[n0] | flags[n0 + 1] << 8 : *reinterpret_cast<const unsigned short *>(flags + n0);
+        // (the caller's marks may begin at any address)
+        const bool bytes = ODD || (reinterpret_cast<size_t>(flags) & 1);
+        const unsigned fw = bytes ? flags[n0] | flags[n0 + 1] << 8 : *reinterpret_cast<const unsigned short *>(flags + n0);
         if (fw & (FL_SOLID | FL_BOUNDARY)) act &= ~1;
         if ((fw >> 8) & (FL_SOLID | FL_BOUNDARY)) act &= ~2;
         if (!act) return;
