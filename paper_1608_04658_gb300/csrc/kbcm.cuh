@@ -75,8 +75,8 @@ __device__ __forceinline__ bool has_stabilizer(double hh, double rho)
     return hh > gamma_floor<double>() * (8.0 / 27.0) * rho && hh > 2.3e-308;
 }
 
-// Root of Eq. (gamma_min) per lane from the analytic value gam (see
-// exact_gamma): with x_i = f'_i(gam)/f^eq_i - 1 and t_i = b dh_i/f'_i(gam),
+// Root of Eq. (gamma_min) per lane (of those in has) from the analytic value gam
+// (see exact_gamma): with x_i = f'_i(gam)/f^eq_i - 1 and t_i = b dh_i/f'_i(gam),
 //   r(gam + s) = sum dh_i log(1 + x_i) - s sum dh_i t_i - s^2/2 sum dh_i t_i^2 - ...,
 // all three sums in one pass (log(1 + x) and 1/(1 + x) by their Taylor series to
 // x^6 and x^3, |x| <= 1/16: truncated below FP32's rounding, the second only
@@ -88,7 +88,7 @@ __device__ __forceinline__ bool has_stabilizer(double hh, double rho)
 template <typename O>
 __device__ __forceinline__ int exact_stabilizer(const typename O::V (&d)[Q], const Shear<typename O::V> &S,
                                                  typename O::V rho, const AxisV<O> &X, const AxisV<O> &Y,
-                                                 const AxisV<O> &Z, typename O::V hh, typename O::R beta,
+                                                 const AxisV<O> &Z, int has, typename O::R beta,
                                                  typename O::R (&gam)[sizeof(typename O::V) / sizeof(typename O::R)])
 {
     using V = typename O::V;
@@ -143,7 +143,7 @@ __device__ __forceinline__ int exact_stabilizer(const typename O::V (&d)[Q], con
     int again = 0;
 #pragma unroll
     for (int k = 0; k < NL; ++k) {
-        if (!has_stabilizer(O::lane(hh, k), O::lane(rho, k))) continue;
+        if (!(has >> k & 1)) continue;
         const R f0 = O::lane(r0, k), f1 = O::lane(r1, k), f2 = O::lane(r2, k), i1 = rcp_fast(f1);
         const R s1 = f0 * i1;
         const R s = s1 - R(0.5) * f2 * s1 * s1 * rcp_fast(f1 + f2 * s1);
@@ -299,17 +299,19 @@ __device__ __forceinline__ int kbc_collide_m(typename O::V (&g)[Q], typename O::
     }
     // stabilizer per node
     R gam[NL], c1v[NL], c2v[NL];
+    int has = 0;  // (for the exact stabilizer, in place of the products)
 #pragma unroll
     for (int k = 0; k < NL; ++k) {
         const R shk = O::lane(sh, k), hhk = O::lane(hh, k);
         gam[k] = R(2);
-        if (gamma_mode != LBM_GAMMA_LBGK && has_stabilizer(hhk, O::lane(rho, k)))
+        if (EXACT) has |= has_stabilizer(hhk, O::lane(rho, k)) << k;
+        if (gamma_mode != LBM_GAMMA_LBGK && (EXACT ? (has >> k & 1) != 0 : has_stabilizer(hhk, O::lane(rho, k))))
             gam[k] = O1<R>::sub(inv_beta, O1<R>::mul(O1<R>::mul(O1<R>::sub(R(2), inv_beta), shk), rcp_fast(hhk)));
     }
     if constexpr (EXACT) {
         if (gamma_mode == LBM_GAMMA_EXACT) {
             const Shear<V> S{sx, sy, sz, qxy, qxz, qyz};
-            ok |= exact_stabilizer<O>(g, S, rho, X, Y, Z, hh, beta, gam) << NL;
+            ok |= exact_stabilizer<O>(g, S, rho, X, Y, Z, has, beta, gam) << NL;
         }
     }
 #pragma unroll
